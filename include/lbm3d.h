@@ -57,7 +57,7 @@ typedef struct {
 
 /* The paper's network: w1[300][19], b1[300], w2[300][300], b2[300],
  * w3[100][300], b3[100], w4[19][100], b4[19], row-major [out][in], device
- * pointers, FP32 (dtype 0).  Read at launch, not copied. */
+ * pointers, FP32 (dtype 0).  Read by every call, not retained. */
 typedef struct {
   const void *w1, *b1, *w2, *b2, *w3, *b3, *w4, *b4;
   int dtype;
@@ -73,7 +73,8 @@ void lbm3d_lattice(int *cx, int *cy, int *cz, float *w);
 /* Create a context over two caller-owned device buffers of
  * 19*nx*ny*nz*batch floats each (ping-pong state) on `cuda_stream` (a
  * cudaStream_t, NULL = default stream) of the current device.  Allocates the
- * status flag and the force tables.  LBM_ERR_ARG on bad parameters. */
+ * status flag, 574 KB of weight scratch for LBM_MLP_F32 and the force tables.
+ * LBM_ERR_ARG on bad parameters. */
 int lbm3d_init(lbm3d_ctx **out, const lbm3d_params *p, float *f_buf0, float *f_buf1,
                void *cuda_stream);
 void lbm3d_destroy(lbm3d_ctx *ctx);
@@ -88,7 +89,8 @@ int lbm3d_init_equilibrium(lbm3d_ctx *ctx, const float *rho, const float *u);
 
 /* Advance n >= 0 steps: pull-stream (Eq. S2), collide with `kind`, EDM force,
  * store.  Both learned kinds take FP32 weights (dtype 0):
- *   LBM_MLP_F32   the network in FP32 on the CUDA cores;
+ *   LBM_MLP_F32   the network in FP32 on the CUDA cores, from a copy of the
+ *                 weights in operand layout refreshed at every call;
  *   LBM_MLP_BF16  the network on the tensor cores (tcgen05): weights, biases
  *                 and activations rounded to bf16, FP32 accumulation; the
  *                 populations, equilibrium, conservation layer and update

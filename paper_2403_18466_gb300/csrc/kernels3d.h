@@ -29,10 +29,15 @@ struct Mlp3 {
 // d3q19_step.cu
 cudaError_t launch_step(const Grid3 &g, const float *in, float *out, const Collide3 &c, int kind,
                         int *flag, cudaStream_t s);
-size_t mlp_f32_smem_bytes();
-cudaError_t launch_step_mlp_f32(const Grid3 &g, const float *in, float *out, const Collide3 &c,
-                                const Mlp3 &w, int *flag, cudaStream_t s);
 cudaError_t launch_set_state(const Grid3 &g, const float *f_pre, float *state, cudaStream_t s);
+
+// d3q19_mlp_f32.cu: the FP32 learned collision.  The weights are first
+// transposed and padded into a device buffer of mlp_f32_weight_floats() floats
+// (16-byte aligned), which the step kernel streams.
+size_t mlp_f32_weight_floats();
+cudaError_t launch_prepare_weights_f32(const Mlp3 &w, float *p, cudaStream_t s);
+cudaError_t launch_step_mlp_f32(const Grid3 &g, const float *in, float *out, const Collide3 &c,
+                                const float *p, int *flag, cudaStream_t s);
 
 // d3q19_mlp_tc.cu: the tensor-core learned collision.  The FP32 weights are
 // first laid out as BF16 operand tiles in a device buffer of

@@ -22,6 +22,7 @@ struct lbm3d_ctx {
   cudaStream_t stream;
   Collide3 cp;
   int *d_flag;     // [0] unstable, [1] device wait timeout
+  float *d_wf32;   // transposed weights of the FP32 collision, in the allocation of d_flag
   float *d_force;  // ny + nz + nx floats (F_x(y), F_y(z), F_z(x)), or nullptr
   void *d_wtc;     // BF16 operand tiles of the tensor-core collision (first use)
   int sms;
@@ -105,12 +106,16 @@ int lbm3d_init(lbm3d_ctx **out, const lbm3d_params *p, float *b0, float *b1, voi
     delete c;
     return LBM_ERR_CUDA;
   }
-  if (cudaMalloc(&c->d_flag, 2 * sizeof(int)) != cudaSuccess ||
+  // flags and the FP32 collision's weight scratch (574 KB) in one allocation,
+  // made here so that a first lbm3d_step may run under stream capture
+  const size_t scratch = 256 + sizeof(float) * lbm::d3::mlp_f32_weight_floats();
+  if (cudaMalloc(&c->d_flag, scratch) != cudaSuccess ||
       cudaMemset(c->d_flag, 0, 2 * sizeof(int)) != cudaSuccess) {
     cudaFree(c->d_flag);
     delete c;
     return LBM_ERR_CUDA;
   }
+  c->d_wf32 = reinterpret_cast<float *>(c->d_flag) + 256 / sizeof(float);
   if (p->force_amp != 0.0) {
     // sine tables in FP64 on the host, one per axis
     std::vector<float> h((size_t)p->ny + p->nz + p->nx);
@@ -171,6 +176,8 @@ int lbm3d_step(lbm3d_ctx *c, int n, lbm_collision kind, const lbm3d_weights *w) 
     if (!c->d_wtc) CUDA_TRY(cudaMalloc(&c->d_wtc, lbm::d3::mlp_tc_weight_bytes()));
     CUDA_TRY(lbm::d3::launch_prepare_weights_tc(f32_view(w), c->d_wtc, c->stream));
   }
+  if (kind == LBM_MLP_F32 && n > 0)
+    CUDA_TRY(lbm::d3::launch_prepare_weights_f32(f32_view(w), c->d_wf32, c->stream));
   for (int s = 0; s < n; ++s) {
     const float *in = c->buf[c->cur];
     float *out = c->buf[c->cur ^ 1];
@@ -178,7 +185,7 @@ int lbm3d_step(lbm3d_ctx *c, int n, lbm_collision kind, const lbm3d_weights *w) 
       CUDA_TRY(lbm::d3::launch_step_mlp_tc(c->g, in, out, c->cp, c->d_wtc, c->sms, c->d_flag,
                                            c->d_flag + 1, c->stream));
     else if (kind == LBM_MLP_F32)
-      CUDA_TRY(lbm::d3::launch_step_mlp_f32(c->g, in, out, c->cp, f32_view(w), c->d_flag,
+      CUDA_TRY(lbm::d3::launch_step_mlp_f32(c->g, in, out, c->cp, c->d_wf32, c->d_flag,
                                             c->stream));
     else
       CUDA_TRY(lbm::d3::launch_step(c->g, in, out, c->cp, kind == LBM_SMAG ? 1 : 0, c->d_flag,
