@@ -7,46 +7,56 @@
 // Per node: x = (f - feq)/rho; h1 = lrelu(W1 x + b1); h2 = lrelu(W2 h1 + b2);
 // h3 = lrelu(W3 h2 + b3); o = W4 h3 + b4; f' = f + (feq - f)/tau + (rho/tau) P o + f_ext.
 //
-// GEMMs per tile of M = 128 nodes (one x row segment), biases folded in as a
-// constant-1 operand column:
+// GEMMs per tile of M = 128 nodes, biases folded in as a constant-1 operand
+// column:
 //   L1  [128 x  32] x [ 32 x 304]   K = 19 inputs + 1 + 12 zeros; N = 300 + 4 zero rows
 //   L2  [128 x 304] x [304 x 304]   K = 300 + 1 + 3 zeros
 //   L3  [128 x 304] x [304 x 112]   N = 100 + 12 zero rows
 //   L4  [128 x 112] x [112 x  32]   K = 100 + 1 + 11 zeros; N = 19 + 13 zero rows
-// N = 304 exceeds one MMA, so L1 and L2 issue two MMAs per K step (N = 160, 144).
+// A tile is 128 consecutive nodes of the flattened lattice (rows, planes and
+// lattices of a batch follow one another), so that narrow lattices fill it.
 //
-// Operands.  The A operands (x and the activations h1, h2, h3, as bf16 pairs)
-// live in tensor memory next to the accumulators: the epilogue reads an
-// accumulator row with tcgen05.ld and writes the activation row back with
-// tcgen05.st, and the next MMA reads A from tensor memory.  That leaves the
-// shared memory to the weights: W1, W3 and W4 stay resident (95 KB); W2
-// (185 KB, which does not fit beside them) is streamed every tile in K chunks
-// of 32 (19,456 bytes) through a 7-slot ring filled by bulk copies
-// (cp.async.bulk) from pre-laid-out copies in global memory (the L2 cache
-// holds them; CTAs read different replicas to spread the L2 traffic).
+// A cluster of two CTAs works on two tiles at a time (cta_group::2, M = 256:
+// each CTA's tensor memory holds its own tile's operands and accumulators, and
+// each CTA's shared memory half of the rows of every weight matrix).  Half of
+// all the weights is 140 KB, so they stay resident for the whole launch; one
+// CTA alone would have to stream W2 (185 KB) again for every tile.
 //
-// Tensor-memory columns: accumulator 0..303, activations (A) 304..455,
-// layer-4 output 456..487, x (layer-1 A) 488..503.
+// N = 304 exceeds one MMA: L1 and L2 run as two passes, columns 0..159 and
+// 160..303.  The A operands (x and the activations, as bf16 pairs) live in
+// tensor memory next to the accumulators: the epilogue reads an accumulator
+// row with tcgen05.ld and writes the activation row back with tcgen05.st.
+// Columns of the tensor memory:
+//     0..303  accumulator of L1 and L2; h2 replaces L2's in place
+//   304..455  h1; then L3's accumulator (304..415), where h3 replaces it
+//   456..487  layer-4 output          488..503  x
+// h1 takes the K steps' columns in an order (H1_RUNS) in which the lower half
+// avoids those h3 of the previous tile still occupies.
 //
-// Roles in a CTA of 320 threads (one CTA per SM, persistent over a contiguous
-// range of tiles):
-//   warps 0-3  (WG0)  the epilogue of the low accumulator columns, and the
-//                     final update and store of each tile (pull, moments,
-//                     conservation layer, BGK, force), done while the next
-//                     tile's second GEMM runs;
-//   warps 4-7  (WG1)  the epilogue of the high accumulator columns, and the
-//                     next tile's layer-1 operand (pull, moments, x), written
-//                     while the current tile's third GEMM runs;
-//   warp 8            MMA issue (one thread);
-//   warp 9            W2 ring producer (one thread).
-// Hand-offs are mbarriers: x ready (128 arrivals), A ready (256 arrivals), the
-// hidden accumulator ready and the output accumulator ready (MMA commits), and
-// the ring's full/empty pairs.  The layer-4 output and x have their own
-// tensor-memory columns, so the next tile's first GEMMs run while the output
-// is read.  Every wait is bounded; on a time-out the kernel records it in
-// shared memory, all roles leave their loops, in-flight copies and MMAs are
-// drained with bounded waits, the tensor memory is freed and the timeout flag
-// is set.
+// What overlaps: L2's first pass starts when the lower half of h1 is written;
+// the lower half of h2 is written while the second pass runs and the upper
+// half while L3 consumes the lower one; the next tile's x, the final update of
+// the previous tile and the pulls of the next one run beside all of that.
+//
+// What bounds it: the MMAs cost ~95 cycles each (N = 160 is at the tensor rate,
+// N = 112 and 32 below it), 68 per tile; the rest of a tile's ~9.6 k cycles is
+// the hop from L3 over L1 to L2 (a commit reaches its waiters ~700 cycles after
+// the last MMA) and the drains, which share the tensor memory with the MMAs.
+// Measured (GB300): 4.0 G nodes/s at 128^3 and 192^3 (1,020 TFLOP/s), 3.56 at
+// 64^3, where one CTA per tile of a row with W2 streamed ran at 2.68, 2.05 and
+// 1.29 G nodes/s.
+//
+// Roles in a CTA of 480 threads (one CTA per SM, a cluster persistent over a
+// contiguous range of tile pairs):
+//   warps 0-3, 4-7 (WG0, WG1)  the epilogues, each half of the columns of each part
+//   warps 8-11     (WG2)       node work: pulls, the layer-1 operand, the final
+//                              update (conservation layer, BGK, force) and store
+//   warps 12-14                MMA issue for both CTAs (one thread each of CTA 0)
+// Hand-offs are mbarriers: the issuers' (x and A operands ready, output read;
+// one arrival per warp of both CTAs, at CTA 0) and the MMA commits', which
+// arrive in both CTAs.  Every wait is bounded; on a time-out the role records
+// it in both CTAs, all roles leave their loops, MMAs in flight are drained
+// with a bounded wait, the tensor memory is freed and the timeout flag is set.
 #include <cuda_bf16.h>
 
 #include "d3q19.cuh"
@@ -61,128 +71,207 @@ using namespace umma;
 
 constexpr int KX = 32;     // layer-1 K
 constexpr int NH = 304;    // padded hidden width (rows of W1, W2 as B operands)
+constexpr int NLO = 160, NHI = NH - NLO;  // the two passes of L1 and L2
 constexpr int KH = 304;    // K of layers 2 and 3
 constexpr int N3 = 112;    // rows of W3
 constexpr int K4 = 112;    // K of layer 4
 constexpr int N4 = 32;     // rows of W4
-constexpr int KC = 32;     // K per streamed W2 chunk
-constexpr int NCHUNK = 10; // 9 chunks of 32 + 1 of 16
-constexpr int SLOTS = 7;
-constexpr int SLOT_BYTES = NH * KC * 2;  // 19,456
-constexpr int W1_BYTES = NH * KX * 2;    // 19,456
-constexpr int W4_BYTES = N4 * K4 * 2;    // 7,168
-constexpr int W3_BYTES = N3 * KH * 2;    // 68,096
-constexpr int W2_CHUNK = NH * KC * 2;    // 19,456 (the last chunk uses half)
-// one pre-laid-out copy of the weights in global memory (bytes)
-constexpr int G_W1 = 0;
-constexpr int G_W4 = G_W1 + W1_BYTES;
-constexpr int G_W3 = G_W4 + W4_BYTES;
-constexpr int G_W2 = G_W3 + W3_BYTES;
-constexpr int G_BYTES = G_W2 + NCHUNK * W2_CHUNK;  // 289,280 per copy
-// Every CTA streams the same 185 KB per tile; REPLICAS copies at different
-// addresses spread the reads over the L2 cache (CTA b reads copy b % REPLICAS).
-constexpr int REPLICAS = 8;
+// one CTA's half of the weights: of each pass, half of the rows
+constexpr int R_LO = NLO / 2, R_HI = NHI / 2, R_H = R_LO + R_HI;
+constexpr int W1_BYTES = R_H * KX * 2;
+constexpr int W2_BYTES = R_H * KH * 2;
+constexpr int W3_BYTES = N3 / 2 * KH * 2;
+constexpr int W4_BYTES = N4 / 2 * K4 * 2;
+constexpr int G_W1 = 0, G_W2 = G_W1 + W1_BYTES, G_W3 = G_W2 + W2_BYTES, G_W4 = G_W3 + W3_BYTES;
+constexpr int G_BYTES = G_W4 + W4_BYTES;  // 139,776 per CTA of the pair
+static_assert(R_LO % 8 == 0 && R_HI % 8 == 0 && G_BYTES % 16 == 0, "operand halves");
 
 // tensor-memory columns
-constexpr uint32_t TM_ACC = 0, TM_A = 304, TM_OUT = 456, TM_X = 488;
+constexpr uint32_t TM_P = 0, TM_A = 304, TM_OUT = 456, TM_X = 488;
+// First column of K step s (16 inputs, 8 columns) of h1, h2 and h3, as packed
+// tables of 6-bit entries (columns / 8), so that the issue loops stay small.
+struct ColTable {
+  uint64_t lo, hi;  // K steps 0..9, 10..18
+  __host__ __device__ constexpr uint32_t operator()(int s) const {
+    return 8u * (uint32_t)(((s < 10 ? lo : hi) >> (6 * (s < 10 ? s : s - 10))) & 63u);
+  }
+};
+struct Run {
+  int k0, n, col;  // K steps k0 .. k0 + n - 1 at col, col + 8, ...
+};
+template <int N>
+constexpr ColTable make_table(const Run (&runs)[N]) {
+  ColTable t{0, 0};
+  for (int r = 0; r < N; ++r)
+    for (int i = 0; i < runs[r].n; ++i) {
+      const int s = runs[r].k0 + i;
+      const uint64_t v = (uint64_t)(runs[r].col / 8 + i);
+      if (s < 10) t.lo |= v << (6 * s);
+      else t.hi |= v << (6 * (s - 10));
+    }
+  return t;
+}
+// the runs of the epilogues' parts: (WG0 | WG1) x (lower | upper), two runs each
+constexpr Run H1_RUNS[8] = {{0, 4, 336},  {4, 1, 416},  {5, 3, 392},  {8, 2, 424},
+                            {10, 4, 304}, {14, 1, 440}, {15, 3, 368}, {18, 1, 448}};
+constexpr Run H2_RUNS[4] = {{0, 5, 0}, {5, 5, 80}, {10, 5, 160}, {15, 4, 240}};
+constexpr Run H3_RUNS[2] = {{0, 4, 304}, {4, 3, 368}};
+constexpr ColTable T1 = make_table(H1_RUNS), T2 = make_table(H2_RUNS), T3 = make_table(H3_RUNS);
+__device__ __forceinline__ ColTable col_h1() { return ColTable{T1.lo, T1.hi}; }
+__device__ __forceinline__ ColTable col_h2() { return ColTable{T2.lo, T2.hi}; }
+__device__ __forceinline__ ColTable col_h3() { return ColTable{T3.lo, T3.hi}; }
 
-constexpr int THREADS = 320;
-constexpr int MMA_WARP = 8, PROD_WARP = 9;
-constexpr uint32_t WAIT_LIMIT = 1u << 22;
+constexpr int TILE = 128;
+constexpr int NODE_WARP = 8, MMA_WARP = 12;
+constexpr int THREADS = 32 * (MMA_WARP + 3);
+// bounded waits: polls, each suspended for at most POLL_NS (1 s in all)
+constexpr uint32_t WAIT_LIMIT = 1u << 18, POLL_NS = 4000;
 
 struct __align__(1024) Smem {
-  unsigned char w1[W1_BYTES];
-  unsigned char w4[W4_BYTES];
-  unsigned char w3[W3_BYTES];
-  unsigned char ring[SLOTS][SLOT_BYTES];
-  unsigned long long full[SLOTS], empty[SLOTS];
-  unsigned long long xready, aready, accready, outready, drain;
+  unsigned char w[G_BYTES];
+  // the issuers' barriers (those of CTA 0 are used): x, halves of h1 and h2, h3, output read
+  unsigned long long bx, b1lo, b1hi, b2lo, b2hi, b3, bo;
+  // MMA commits (both CTAs'): L1 and L2 (two passes each), L3, L4
+  unsigned long long c1a, c1b, c2a, c2b, c3, c4;
+  unsigned long long wload, drain[3];
   uint32_t taddr;
   int err;
 };
 constexpr size_t SMEM_BYTES = sizeof(Smem) + 1024;
 static_assert(SMEM_BYTES <= 232448, "shared memory layout too large");
 
-__host__ __device__ constexpr int chunk_k(int c) {
-  return c < NCHUNK - 1 ? KC : KH - KC * (NCHUNK - 1);
-}
-
 // ---- helpers ------------------------------------------------------------------
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
 }
-// Non-blocking test of a phase (mbarrier.test_wait never suspends the thread,
-// so a completed phase is seen at the next poll).
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
 }
-// Bounded wait that also gives up early once another role has recorded an
-// error.  Polls back off with a short sleep so that waiting warps leave the
-// issue slots to the warps that work.
-template <bool SLEEP = true>
-__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volatile int *err) {
+// Shared-memory address of the same variable in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_cta(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// Arrivals and waits order tensor-memory accesses only (through the tcgen05
+// fences around them), no generic memory, so they need no cluster-wide
+// release or acquire: those cost ~1,000 and ~400 cycles each.
+__device__ __forceinline__ void arrive_cluster(uint32_t mapped) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(mapped) : "memory");
+}
+__device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
+  return mbar_try_wait_sleep(bar, parity, POLL_NS);
+}
+// A time-out: both CTAs' roles see it at their next wait.
+__device__ __forceinline__ void record_error(int *err) {
+  const uint32_t a = smem_u32(err);
+  for (uint32_t k = 0; k < 2; ++k)
+    asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(map_cta(a, k)), "r"(1)
+                 : "memory");
+}
+// Bounded wait that only the limit ends early (copies and MMAs in flight).
+__device__ __forceinline__ bool wait_done(uint32_t bar) {
+  return mbar_wait_sleep_bounded(bar, 0, WAIT_LIMIT, POLL_NS);
+}
+// Bounded wait that also gives up early once a role has recorded an error.
+__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, int *err) {
   for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
-    if (mbar_test(bar, parity)) return true;
-    if ((it & 63u) == 63u && *err) return false;
-    if (SLEEP) __nanosleep(20);
+    if (try_wait(bar, parity)) return true;
+    if ((it & 63u) == 63u && *reinterpret_cast<volatile int *>(err)) return false;
   }
-  atomicOr(const_cast<int *>(err), 1);
+  record_error(err);
   return false;
 }
 // The same for a whole warp: every lane waits in mbarrier.try_wait (the
 // hardware suspends the warp until the phase completes or a short time limit
 // passes) and the lanes agree by a vote, so the warp stays converged for the
 // .sync.aligned tensor-memory accesses that follow and waiting warps take no
-// issue slots from the MMA and producer warps.  (Lane 0 polling test_wait with
-// the other lanes held at a shuffle cost 10 % of the step: 2.46 against
-// 2.73 G nodes/s at 256^3.)
-__device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, volatile int *err) {
+// issue slots from the MMA warp.  (Lane 0 polling test_wait with the other
+// lanes held at a shuffle cost 10 % of the step.)
+__device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, int *err) {
   for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
-    if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    if ((it & 63u) == 63u && __any_sync(0xffffffffu, *err != 0)) return false;
+    if (__any_sync(0xffffffffu, try_wait(bar, parity))) {
+      fence_after_sync();
+      return true;
+    }
+    if ((it & 63u) == 63u &&
+        __any_sync(0xffffffffu, *reinterpret_cast<volatile int *>(err) != 0))
+      return false;
   }
-  if ((threadIdx.x & 31) == 0) atomicOr(const_cast<int *>(err), 1);
+  if ((threadIdx.x & 31) == 0) record_error(err);
   return false;
 }
-// D (+)= A[tmem] * B[smem]^T, one elected thread.
-__device__ __forceinline__ void mma_ta(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t id,
-                                       bool acc) {
+// After this warp's tensor-memory accesses: one arrival at CTA 0's barrier.
+__device__ __forceinline__ void publish(uint32_t mapped) {
+  tmem_wait_st();
+  fence_before_sync();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) arrive_cluster(mapped);
+}
+// Both CTAs' D (+)= A[tmem] * B[smem halves]^T, one thread of CTA 0.
+__device__ __forceinline__ void mma_pair(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t id,
+                                         bool acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
       "r"(a_tmem), "l"(b), "r"(id), "r"(acc ? 1u : 0u)
       : "memory");
 }
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) { return pack_bf16x2(lo, hi); }
-__device__ __forceinline__ float lrelu(float v) { return fmaxf(v, LEAKY * v); }
+// Arrive on this barrier of both CTAs when the MMAs issued so far are done.
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+      "[%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
 
-// Tile walk: 128 consecutive x of row (b, z, y).
-struct Tile {
-  int b, z, y, x0;
-  __device__ __forceinline__ void set(int t, int tiles_x, int ny, int nz) {
-    x0 = (t % tiles_x) * 128;
-    int row = t / tiles_x;
-    y = row % ny;
-    row /= ny;
-    z = row % nz;
-    b = row / nz;
-  }
+// A node of the flattened lattice, walked in steps of two tiles.
+struct NodePos {
+  long long n;
+  int x, y, z, b;
 };
+struct NodeStep {
+  int dx, dy, dz, db;
+};
+__device__ __forceinline__ NodePos locate(const Grid3 &g, long long n) {
+  NodePos p;
+  p.n = n;
+  long long row = n / g.nx;
+  p.x = (int)(n - row * g.nx);
+  long long pl = row / g.ny;
+  p.y = (int)(row - pl * g.ny);
+  p.b = (int)(pl / g.nz);
+  p.z = (int)(pl - (long long)p.b * g.nz);
+  return p;
+}
+__device__ __forceinline__ void advance(NodePos &p, const Grid3 &g, const NodeStep &d) {
+  p.n += 2 * TILE;
+  p.x += d.dx;
+  int c = p.x >= g.nx;
+  p.x -= c ? g.nx : 0;
+  p.y += d.dy + c;
+  c = p.y >= g.ny;
+  p.y -= c ? g.ny : 0;
+  p.z += d.dz + c;
+  c = p.z >= g.nz;
+  p.z -= c ? g.nz : 0;
+  p.b += d.db + c;
+}
 
-__device__ __forceinline__ void pull19(const float *__restrict__ in, const Grid3 &g, const Tile &T,
-                                       int x, float d[Q]) {
+__device__ __forceinline__ void pull19(const float *__restrict__ in, const Grid3 &g,
+                                       const NodePos &p, long long nodes, float d[Q]) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) d[i] = 0.f;
+  if (p.n >= nodes) return;
   const size_t vol = g.volume();
-  const float *gb = in + (size_t)T.b * Q * vol;
+  const float *gb = in + (size_t)p.b * Q * vol;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    int xs = x - cx(i), ys = T.y - cy(i), zs = T.z - cz(i);
+    int xs = p.x - cx(i), ys = p.y - cy(i), zs = p.z - cz(i);
     xs = xs < 0 ? xs + g.nx : (xs >= g.nx ? xs - g.nx : xs);
     ys = ys < 0 ? ys + g.ny : (ys >= g.ny ? ys - g.ny : ys);
     zs = zs < 0 ? zs + g.nz : (zs >= g.nz ? zs - g.nz : zs);
@@ -190,58 +279,41 @@ __device__ __forceinline__ void pull19(const float *__restrict__ in, const Grid3
   }
 }
 
-// Drain NCOL accumulator columns starting at C0 of this thread's row (loads
-// issued before one wait): LeakyReLU, bf16 pairs, into activation columns
-// TM_A + C0/2 of the same row.  Columns at or above KVALID are not
-// activations: KVALID gets the constant 1 (the bias column), the rest zero.
-template <int C0, int NCOL, int KVALID>
-__device__ __forceinline__ void drain_cols(uint32_t tm_row) {
-  static_assert(NCOL % 16 == 0 && NCOL <= 64, "16..64 columns per drain");
-  uint32_t v[NCOL];
+// 16 accumulator columns -> LeakyReLU -> 8 columns of bf16 pairs.  The two
+// products 0.01 v of a pair in one packed multiply (round to nearest per lane,
+// as the scalar form), then max.
+__device__ __forceinline__ void activate16(const uint32_t (&v)[16], uint32_t dst) {
+  uint32_t p[8];
 #pragma unroll
-  for (int q = 0; q < NCOL / 16; ++q)
-    tmem_ld16(tm_row + (uint32_t)(TM_ACC + C0 + 16 * q),
-              *reinterpret_cast<uint32_t(*)[16]>(v + 16 * q));
-  tmem_wait_ld();
-  uint32_t p[NCOL / 2];
-#pragma unroll
-  for (int e = 0; e < NCOL / 2; ++e) {
-    const int k = C0 + 2 * e;
-    if (k + 1 < KVALID) {
-      // LeakyReLU of both values: the two products 0.01 v in one packed
-      // multiply (round to nearest per lane, as the scalar form), then max
-      const float a0 = __uint_as_float(v[2 * e]), a1 = __uint_as_float(v[2 * e + 1]);
-      const float2 s = __fmul2_rn(make_float2(a0, a1), make_float2(LEAKY, LEAKY));
-      p[e] = pack2(fmaxf(a0, s.x), fmaxf(a1, s.y));
-    } else {
-      float h[2];
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-        h[j] = k + j < KVALID ? lrelu(__uint_as_float(v[2 * e + j]))
-                              : (k + j == KVALID ? 1.0f : 0.0f);
-      p[e] = pack2(h[0], h[1]);
-    }
+  for (int e = 0; e < 8; ++e) {
+    const float a0 = __uint_as_float(v[2 * e]), a1 = __uint_as_float(v[2 * e + 1]);
+    const float2 s = __fmul2_rn(make_float2(a0, a1), make_float2(LEAKY, LEAKY));
+    p[e] = pack_bf16x2(fmaxf(a0, s.x), fmaxf(a1, s.y));
   }
-#pragma unroll
-  for (int q = 0; q < NCOL / 32; ++q)
-    tmem_st16(tm_row + (uint32_t)(TM_A + C0 / 2 + 16 * q),
-              *reinterpret_cast<const uint32_t(*)[16]>(p + 16 * q));
-  if (NCOL % 32)
-    tmem_st8(tm_row + (uint32_t)(TM_A + C0 / 2 + 16 * (NCOL / 32)),
-             *reinterpret_cast<const uint32_t(*)[8]>(p + 16 * (NCOL / 32)));
+  tmem_st8(dst, p);
 }
-
-// The low (WG0) or high (WG1) half of a 304-column accumulator -> h (K 0..303).
-__device__ __forceinline__ void drain_hidden(int wg, uint32_t tm_row) {
-  if (wg == 0) {
-    drain_cols<0, 64, H1>(tm_row);
-    drain_cols<64, 64, H1>(tm_row);
-    drain_cols<128, 32, H1>(tm_row);
-  } else {
-    drain_cols<160, 64, H1>(tm_row);
-    drain_cols<224, 64, H1>(tm_row);
-    drain_cols<288, 16, H1>(tm_row);
-  }
+// K steps k0 .. k0 + steps - 1 (3 to 5) of a layer's accumulator (from tensor-
+// memory column acc on) -> activations at the columns `table` gives.  All
+// loads are issued before one wait, so in-place stores follow the loads of the
+// columns they replace.  The padding needs no special case: the row after a
+// layer's last unit in the prepared weights has its bias 1 and all else 0, so
+// its accumulator is the constant input of the next layer, and the rows after
+// it are 0.
+// One body serves all layers and both warpgroups: a drain compiled for each
+// part made the kernel 100 KB long, and most SMs then waited for instructions
+// (13.6 k cycles per tile against 9.4 k on the few that did not).
+__device__ __forceinline__ void drain(uint32_t tm_row, uint32_t acc, const ColTable &table, int k0,
+                                      int steps) {
+  uint32_t v[5][16];
+  const uint32_t src = tm_row + acc + 16 * k0;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) tmem_ld16(src + 16 * s, v[s]);
+  if (steps > 3) tmem_ld16(src + 48, v[3]);
+  if (steps > 4) tmem_ld16(src + 64, v[4]);
+  tmem_wait_ld();
+#pragma unroll
+  for (int s = 0; s < 5; ++s)
+    if (s < 3 || steps > s) activate16(v[s], tm_row + table(k0 + s));
 }
 
 // x = (f - feq)/rho of this thread's node -> its row of the layer-1 operand
@@ -257,334 +329,316 @@ __device__ __forceinline__ void write_x(const float d[Q], bool active, uint32_t 
     xi[i] = i < Q ? (active ? (d[i] - deq[i]) * inv_rho : 0.f) : (i == Q ? 1.0f : 0.0f);
   uint32_t p[16];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) p[e] = pack2(xi[2 * e], xi[2 * e + 1]);
+  for (int e = 0; e < 16; ++e) p[e] = pack_bf16x2(xi[2 * e], xi[2 * e + 1]);
   tmem_st16(tm_row + TM_X, p);
 }
 
-// Arrive on `bar` after this thread's tensor-memory stores are complete.
-__device__ __forceinline__ void publish(uint32_t bar) {
-  tmem_wait_st();
-  fence_before_sync();
-  mbar_arrive(bar);
-}
-
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     k3_step_mlp_tc(const float *__restrict__ in, float *__restrict__ out, Grid3 g, Collide3 cp,
                    const unsigned char *__restrict__ gw, int *flag, int *timeout_flag) {
   extern __shared__ unsigned char smem_raw[];
   Smem &S = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                       ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  volatile int *err = &S.err;
-  gw += (size_t)(blockIdx.x % REPLICAS) * G_BYTES;
+  const uint32_t rank = cluster_rank();
+  int *err = &S.err;
 
-  // ---- prologue: resident weights, barriers, tensor memory
-  {
-    const uint4 *src = reinterpret_cast<const uint4 *>(gw + G_W1);
-    uint4 *dst = reinterpret_cast<uint4 *>(S.w1);
-    for (int e = tid; e < W1_BYTES / 16; e += THREADS) dst[e] = src[e];
-    src = reinterpret_cast<const uint4 *>(gw + G_W4);
-    dst = reinterpret_cast<uint4 *>(S.w4);
-    for (int e = tid; e < W4_BYTES / 16; e += THREADS) dst[e] = src[e];
-    src = reinterpret_cast<const uint4 *>(gw + G_W3);
-    dst = reinterpret_cast<uint4 *>(S.w3);
-    for (int e = tid; e < W3_BYTES / 16; e += THREADS) dst[e] = src[e];
-  }
+  // ---- prologue: barriers, this CTA's half of the weights, tensor memory
   if (tid == 0) {
-    for (int s = 0; s < SLOTS; ++s) {
-      mbar_init(smem_u32(&S.full[s]), 1);
-      mbar_init(smem_u32(&S.empty[s]), 1);
-    }
-    mbar_init(smem_u32(&S.xready), 128);
-    mbar_init(smem_u32(&S.aready), 256);
-    mbar_init(smem_u32(&S.accready), 1);
-    mbar_init(smem_u32(&S.outready), 1);
-    mbar_init(smem_u32(&S.drain), 1);
+    mbar_init(smem_u32(&S.bx), 8);
+    mbar_init(smem_u32(&S.bo), 8);
+    for (unsigned long long *b : {&S.b1lo, &S.b1hi, &S.b2lo, &S.b2hi, &S.b3})
+      mbar_init(smem_u32(b), 16);
+    for (unsigned long long *b : {&S.c1a, &S.c1b, &S.c2a, &S.c2b, &S.c3, &S.c4, &S.wload, &S.drain[0],
+                                  &S.drain[1], &S.drain[2]})
+      mbar_init(smem_u32(b), 1);
     S.err = 0;
     fence_mbarrier_init();
+    fence_proxy_async();
+    const uint32_t bar = smem_u32(&S.wload);
+    mbar_arrive_expect_tx(bar, G_BYTES);
+    const unsigned char *src = gw + (size_t)rank * G_BYTES;
+    for (int at = 0; at < G_BYTES; at += 16384) {
+      const uint32_t n = G_BYTES - at < 16384 ? G_BYTES - at : 16384;
+      bulk_g2s(smem_u32(S.w) + at, src + at, n, bar);
+    }
   }
   if (warp == 0) {
-    tmem_alloc(smem_u32(&S.taddr), 512);
-    tmem_relinquish();
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                     smem_u32(&S.taddr))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  fence_proxy_async();
   fence_before_sync();
   __syncthreads();
+  // the weights have landed (bounded; every thread polls, so that all see the copy)
+  if (!wait_done(smem_u32(&S.wload))) S.err = 1;
+  cluster_sync();
   fence_after_sync();
   const uint32_t tmem = S.taddr;
+  // the prologue reads only the prepared weights: launched as a programmatic
+  // dependent of the previous step, it waits for that step here
+  griddep_wait();
+  griddep_launch_dependents();
 
-  // ---- this CTA's contiguous range of tiles
-  const int tiles_x = (g.nx + 127) / 128;
-  const int ntiles = (int)((long long)tiles_x * g.ny * g.nz * g.batch);
-  const int per = ntiles / gridDim.x, extra = ntiles % gridDim.x;
-  const int t_begin = blockIdx.x * per + min((int)blockIdx.x, extra);
-  const int count = per + ((int)blockIdx.x < extra ? 1 : 0);
+  // ---- this cluster's contiguous range of tile pairs
+  const long long nodes = (long long)g.nx * g.ny * g.nz * g.batch;
+  const long long pairs = (nodes + 2 * TILE - 1) / (2 * TILE);
+  const int clusters = gridDim.x / 2, cid = blockIdx.x / 2;
+  const long long per = pairs / clusters, extra = pairs % clusters;
+  const long long p_begin = cid * per + (cid < extra ? cid : extra);
+  const int count = (int)(per + (cid < extra ? 1 : 0));
+  const bool ok0 = *reinterpret_cast<volatile int *>(err) == 0;
 
-  if (warp == PROD_WARP) {
-    // ---------------- W2 ring producer
-    if (lane == 0) {
-      uint32_t used_mask = 0, par_mask = 0;  // per slot: used once; parity of its next use
-      int slot = 0;
-      bool ok = true;
-      for (int t = 0; t < count && ok; ++t) {
-        for (int c = 0; c < NCHUNK; ++c) {
-          const uint32_t full = smem_u32(&S.full[slot]), empty = smem_u32(&S.empty[slot]);
-          const uint32_t bit = 1u << slot;
-          // the previous use of this slot must have been consumed
-          if ((used_mask & bit) && !wait_phase(empty, (par_mask & bit) ? 0u : 1u, err)) {
-            ok = false;
-            break;
-          }
-          const uint32_t bytes = (uint32_t)(NH * chunk_k(c) * 2);
-          mbar_arrive_expect_tx(full, bytes);
-          bulk_g2s(smem_u32(S.ring[slot]), gw + G_W2 + c * W2_CHUNK, bytes, full);
-          used_mask |= bit;
-          par_mask ^= bit;
-          slot = slot + 1 == SLOTS ? 0 : slot + 1;
-        }
-      }
-      // drain: every issued copy has landed before the CTA may exit
-      for (int s = 0; s < SLOTS; ++s)
-        if (used_mask & (1u << s)) {
-          const uint32_t full = smem_u32(&S.full[s]);
-          const uint32_t last = (par_mask & (1u << s)) ? 0u : 1u;  // parity of the last use
-          for (uint32_t it = 0; it < WAIT_LIMIT; ++it)
-            if (mbar_test(full, last)) break;
-        }
-    }
-  } else if (warp == MMA_WARP) {
-    // ---------------- MMA issue
-    if (lane == 0) {
-      const uint32_t sw1 = smem_u32(S.w1), sw3 = smem_u32(S.w3), sw4 = smem_u32(S.w4);
-      const uint32_t bar_acc = smem_u32(&S.accready), bar_out = smem_u32(&S.outready);
-      const uint32_t acc = tmem + TM_ACC, ah = tmem + TM_A, ax = tmem + TM_X;
-      constexpr uint32_t ID160 = idesc_bf16_f32(128, 160), ID144 = idesc_bf16_f32(128, 144),
-                         ID112 = idesc_bf16_f32(128, 112), ID32 = idesc_bf16_f32(128, 32);
-      uint32_t px = 0, pa = 0, par_mask = 0;  // par bit s = parity of the slot's next use
-      int slot = 0;
+  if (warp >= MMA_WARP) {
+    // ---------------- MMA issue: L1 and L2, L3, L4 by a thread each.  (A
+    // thread that has committed stalls at its next memory access until its
+    // MMAs have completed, so one thread for all would start every layer that
+    // much late.)
+    if (rank == 0 && lane == 0 && ok0) {
+      const uint32_t sw = smem_u32(S.w);
+      constexpr uint32_t ID_LO = idesc_bf16_f32(256, NLO), ID_HI = idesc_bf16_f32(256, NHI),
+                         ID_3 = idesc_bf16_f32(256, N3), ID_4 = idesc_bf16_f32(256, N4);
+      const uint32_t P = tmem + TM_P;
       bool issued = false;
-      // the first tile's x (later tiles' x is awaited after the L4 commit)
-      bool xok = count > 0 && wait_phase<false>(smem_u32(&S.xready), px, err);
-      px ^= 1;
-      for (int t = 0; t < count && xok; ++t) {
-        // L1: A = x (tensor memory, K 32), B = W1 resident
-        fence_after_sync();
-#pragma unroll
-        for (int s = 0; s < KX / 16; ++s) {
-          mma_ta(acc, ax + 8 * s, smem_desc(sw1 + 256 * s, 128, 16 * KX), ID160, s > 0);
-          mma_ta(acc + 160, ax + 8 * s, smem_desc(sw1 + 20 * 16 * KX + 256 * s, 128, 16 * KX),
-                 ID144, s > 0);
-        }
-        mma_commit(bar_acc);
-        issued = true;
-        // L2: A = h1 (tensor memory, K 304), B = streamed W2 chunks, consumed
-        // as they land (the stream from the L2 cache sets the pace).  Note that
-        // on this GPU the first memory access of a thread after a
-        // tcgen05.commit waits until the MMAs it has issued have completed.
-        if (!wait_phase<false>(smem_u32(&S.aready), pa, err)) break;
-        pa ^= 1;
-        fence_after_sync();
-        bool ok = true;
-        for (int c = 0; c < NCHUNK; ++c) {
-          if (!wait_phase<false>(smem_u32(&S.full[slot]), (par_mask >> slot) & 1u, err)) {
-            ok = false;
+      uint32_t par = 0;  // parity of tile t's events
+      if (warp == MMA_WARP) {
+        const uint32_t w1lo = sw + G_W1, w1hi = w1lo + R_LO * KX * 2;
+        const uint32_t w2lo = sw + G_W2, w2hi = w2lo + R_LO * KH * 2;
+        for (int t = 0; t < count; ++t, par ^= 1) {
+          // L1: its accumulator replaces the previous tile's h2, so that tile's
+          // L3 has to be complete
+          if (!(wait_phase(smem_u32(&S.bx), par, err) &&
+                (t == 0 || wait_phase(smem_u32(&S.c3), par ^ 1, err))))
             break;
-          }
-          par_mask ^= 1u << slot;
-          const int kc = chunk_k(c);
-          const uint32_t sb = smem_u32(S.ring[slot]);
-          for (int s = 0; s < kc / 16; ++s) {
-            const uint32_t a = ah + 8 * (2 * c + s);
-            const bool accum = c > 0 || s > 0;
-            mma_ta(acc, a, smem_desc(sb + 256 * s, 128, 16 * kc), ID160, accum);
-            mma_ta(acc + 160, a, smem_desc(sb + 20 * 16 * kc + 256 * s, 128, 16 * kc), ID144,
-                   accum);
-          }
-          mma_commit(smem_u32(&S.empty[slot]));
-          slot = slot + 1 == SLOTS ? 0 : slot + 1;
+          fence_after_sync();
+#pragma unroll
+          for (int s = 0; s < KX / 16; ++s)
+            mma_pair(P, tmem + TM_X + 8 * s, smem_desc(w1lo + 256 * s, 128, 16 * KX), ID_LO, s > 0);
+          commit_pair(smem_u32(&S.c1a));
+#pragma unroll
+          for (int s = 0; s < KX / 16; ++s)
+            mma_pair(P + NLO, tmem + TM_X + 8 * s, smem_desc(w1hi + 256 * s, 128, 16 * KX), ID_HI,
+                     s > 0);
+          commit_pair(smem_u32(&S.c1b));
+          issued = true;
+          // L2, first pass: the lower half of h1 is ready before the upper one
+          if (!wait_phase(smem_u32(&S.b1lo), par, err)) break;
+          fence_after_sync();
+#pragma unroll
+          for (int s = 0; s < NLO / 16; ++s)
+            mma_pair(P, tmem + col_h1()(s), smem_desc(w2lo + 256 * s, 128, 16 * KH), ID_LO, s > 0);
+          if (!wait_phase(smem_u32(&S.b1hi), par, err)) break;
+          fence_after_sync();
+#pragma unroll
+          for (int s = NLO / 16; s < KH / 16; ++s)
+            mma_pair(P, tmem + col_h1()(s), smem_desc(w2lo + 256 * s, 128, 16 * KH), ID_LO, true);
+          commit_pair(smem_u32(&S.c2a));
+          // second pass
+#pragma unroll
+          for (int s = 0; s < KH / 16; ++s)
+            mma_pair(P + NLO, tmem + col_h1()(s), smem_desc(w2hi + 256 * s, 128, 16 * KH), ID_HI,
+                     s > 0);
+          commit_pair(smem_u32(&S.c2b));
         }
-        if (!ok) break;
-        mma_commit(bar_acc);
-        // L3: A = h2, B = W3 resident (K 304, N 112)
-        if (!wait_phase<false>(smem_u32(&S.aready), pa, err)) break;
-        pa ^= 1;
-        fence_after_sync();
-#pragma unroll 1
-        for (int s = 0; s < KH / 16; ++s)
-          mma_ta(acc, ah + 8 * s, smem_desc(sw3 + 256 * s, 128, 16 * KH), ID112, s > 0);
-        mma_commit(bar_acc);
-        // L4: A = h3 (K 112), B = W4 resident; its own accumulator columns
-        if (!wait_phase<false>(smem_u32(&S.aready), pa, err)) break;
-        pa ^= 1;
-        fence_after_sync();
+      } else if (warp == MMA_WARP + 1) {
+        // L3: its accumulator replaces h1, so L2 has to be complete
+        const uint32_t w3 = sw + G_W3, D3 = tmem + TM_A;
+        for (int t = 0; t < count; ++t, par ^= 1) {
+          if (!(wait_phase(smem_u32(&S.c2b), par, err) && wait_phase(smem_u32(&S.b2lo), par, err)))
+            break;
+          fence_after_sync();
 #pragma unroll
-        for (int s = 0; s < K4 / 16; ++s)
-          mma_ta(tmem + TM_OUT, ah + 8 * s, smem_desc(sw4 + 256 * s, 128, 16 * K4), ID32, s > 0);
-        mma_commit(bar_out);
-        if (t + 1 < count) {  // the next tile's x
-          xok = wait_phase<false>(smem_u32(&S.xready), px, err);
-          px ^= 1;
+          for (int s = 0; s < NLO / 16; ++s)
+            mma_pair(D3, tmem + col_h2()(s), smem_desc(w3 + 256 * s, 128, 16 * KH), ID_3, s > 0);
+          issued = true;
+          if (!wait_phase(smem_u32(&S.b2hi), par, err)) break;
+          fence_after_sync();
+#pragma unroll
+          for (int s = NLO / 16; s < KH / 16; ++s)
+            mma_pair(D3, tmem + col_h2()(s), smem_desc(w3 + 256 * s, 128, 16 * KH), ID_3, true);
+          commit_pair(smem_u32(&S.c3));
         }
-      }
-      // drain outstanding MMAs before the tensor memory is freed
-      if (issued) {
-        mma_commit(smem_u32(&S.drain));
-        for (uint32_t it = 0; it < WAIT_LIMIT; ++it)
-          if (mbar_test(smem_u32(&S.drain), 0)) break;
-      }
-    }
-  } else {
-    // ---------------- node and epilogue warpgroups
-    const int wg = warp >> 2;
-    const int r = tid & 127;
-    const uint32_t tm_row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-    const uint32_t bar_acc = smem_u32(&S.accready), bar_out = smem_u32(&S.outready),
-                   bar_a = smem_u32(&S.aready), bar_x = smem_u32(&S.xready);
-    uint32_t pacc = 0, pout = 0;
-    const size_t vol = g.volume();
-    Tile T;
-    T.set(t_begin, tiles_x, g.ny, g.nz);
-    Tile P = T;  // WG0: the tile whose final update is pending
-    float d[Q];  // WG0: populations of tile P; WG1: of the next tile to prepare
-#pragma unroll
-    for (int i = 0; i < Q; ++i) d[i] = 0.f;
-    if (count > 0 && T.x0 + r < g.nx) pull19(in, g, T, T.x0 + r, d);
-    if (wg == 1 && count > 0) {
-      write_x(d, T.x0 + r < g.nx, tm_row);
-      publish(bar_x);
-    }
-
-    // WG0: final update of tile P from the layer-4 output; then load the
-    // populations of tile `next` (if any) for its own final update.
-    auto finish = [&](const Tile &next, bool have_next) -> bool {
-      const int x = P.x0 + r;
-      const bool active = x < g.nx;
-      const Moments m = node_moments(d);
-      {
-        const unsigned mask = __ballot_sync(0xffffffffu, active && is_unstable(m));
-        if (mask && lane == (__ffs(mask) - 1) && *reinterpret_cast<volatile int *>(flag) == 0)
-          atomicOr(flag, 1);
-      }
-      float deq[Q];
-      shifted_feq(m, deq);
-      if (!wait_phase_warp(bar_out, pout, err)) return false;
-      pout ^= 1;
-      fence_after_sync();
-      uint32_t v0[16], v1[16];
-      tmem_ld16(tm_row + TM_OUT, v0);
-      tmem_ld16(tm_row + TM_OUT + 16, v1);
-      tmem_wait_ld();
-      fence_before_sync();
-      float o[Q];
-#pragma unroll
-      for (int i = 0; i < Q; ++i) o[i] = __uint_as_float(i < 16 ? v0[i] : v1[i - 16]);
-      project(o);
-      if (active) {
-        const float rw = m.rho * cp.omega;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) d[i] = fmaf(cp.omega, deq[i] - d[i], d[i]) + rw * o[i];
-        const float Fx = cp.fx_y ? __ldg(cp.fx_y + P.y) : 0.f;
-        const float Fy = cp.fy_z ? __ldg(cp.fy_z + P.z) : 0.f;
-        const float Fz = cp.fz_x ? __ldg(cp.fz_x + x) : 0.f;
-        add_edm_force(m, Fx, Fy, Fz, d);
-        float *ob = out + (size_t)P.b * Q * vol + ((size_t)P.z * g.ny + P.y) * g.nx + x;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) ob[(size_t)i * vol] = d[i];
-      }
-#pragma unroll
-      for (int i = 0; i < Q; ++i) d[i] = 0.f;
-      if (have_next && next.x0 + r < g.nx) pull19(in, g, next, next.x0 + r, d);
-      P = next;
-      return true;
-    };
-
-    for (int t = 0; t < count; ++t) {
-      Tile N = T;
-      const bool has_next = t + 1 < count;
-      if (has_next) N.set(t_begin + t + 1, tiles_x, g.ny, g.nz);
-      // L1 -> h1
-      if (!wait_phase_warp(bar_acc, pacc, err)) break;
-      pacc ^= 1;
-      fence_after_sync();
-      drain_hidden(wg, tm_row);
-      publish(bar_a);
-      if (wg == 0) {
-        if (t > 0 && !finish(T, true)) break;  // tile t-1 done; tile t's populations loaded
       } else {
-        // the next tile's populations, needed after L2
+        // L4, once the previous tile's output has been read
+        const uint32_t w4 = sw + G_W4;
+        for (int t = 0; t < count; ++t, par ^= 1) {
+          if (!(wait_phase(smem_u32(&S.b3), par, err) &&
+                (t == 0 || wait_phase(smem_u32(&S.bo), par ^ 1, err))))
+            break;
+          fence_after_sync();
 #pragma unroll
-        for (int i = 0; i < Q; ++i) d[i] = 0.f;
-        if (has_next && N.x0 + r < g.nx) pull19(in, g, N, N.x0 + r, d);
+          for (int s = 0; s < K4 / 16; ++s)
+            mma_pair(tmem + TM_OUT, tmem + col_h3()(s), smem_desc(w4 + 256 * s, 128, 16 * K4), ID_4,
+                     s > 0);
+          commit_pair(smem_u32(&S.c4));
+          issued = true;
+        }
       }
-      // L2 -> h2
-      if (!wait_phase_warp(bar_acc, pacc, err)) break;
-      pacc ^= 1;
-      fence_after_sync();
-      drain_hidden(wg, tm_row);
-      publish(bar_a);
-      if (wg == 1 && has_next) {
-        // the next tile's layer-1 operand (L1 of this tile has read x)
-        write_x(d, N.x0 + r < g.nx, tm_row);
-        publish(bar_x);
+      // this thread's outstanding MMAs are done before the tensor memory is freed
+      if (issued) {
+        const uint32_t bar = smem_u32(&S.drain[warp - MMA_WARP]);
+        commit_pair(bar);
+        if (!wait_done(bar)) record_error(err);
       }
-      // L3 -> h3 (K 0..99, the constant column at 100, zeros to 111)
-      if (!wait_phase_warp(bar_acc, pacc, err)) break;
-      pacc ^= 1;
-      fence_after_sync();
-      if (wg == 0)
-        drain_cols<0, 64, H3>(tm_row);
-      else
-        drain_cols<64, 48, H3>(tm_row);
-      publish(bar_a);
-      T = N;
     }
-    // WG0: the last tile's final update
-    if (wg == 0 && count > 0 && !*err) finish(T, false);
+    __syncwarp();
+  } else if (warp >= NODE_WARP) {
+    // ---------------- node work
+    const int r = tid - 32 * NODE_WARP;
+    const uint32_t tm_row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    const uint32_t m_x = map_cta(smem_u32(&S.bx), 0), m_o = map_cta(smem_u32(&S.bo), 0);
+    const uint32_t c1 = smem_u32(&S.c1b), c4 = smem_u32(&S.c4);
+    const size_t vol = g.volume();
+    NodeStep st;
+    {
+      int q = 2 * TILE / g.nx;
+      st.dx = 2 * TILE % g.nx;
+      st.dy = q % g.ny;
+      q /= g.ny;
+      st.dz = q % g.nz;
+      st.db = q / g.nz;
+    }
+    // Iteration t loads tile t + 2, writes the layer-1 operand of tile t + 1 and
+    // finishes tile t (one body for all, for the instruction cache).
+    NodePos P{}, N{}, F = locate(g, p_begin * 2 * TILE + rank * TILE + r);
+    float d[Q], dn[Q], df[Q];  // populations of tiles t, t + 1, t + 2
+#pragma unroll
+    for (int i = 0; i < Q; ++i) d[i] = dn[i] = df[i] = 0.f;
+#pragma unroll 1
+    for (int t = -2; t < count && ok0; ++t) {
+      const uint32_t par = t & 1;
+      if (t + 2 < count) pull19(in, g, F, nodes, df);
+      if (t >= -1 && t + 1 < count) {
+        if (t >= 0 && !wait_phase_warp(c1, par, err)) break;  // L1 has read x
+        write_x(dn, N.n < nodes, tm_row);
+        publish(m_x);
+      }
+      if (t >= 0) {
+        const bool active = P.n < nodes;
+        const Moments m = node_moments(d);
+        {
+          const unsigned mask = __ballot_sync(0xffffffffu, active && is_unstable(m));
+          if (mask && lane == (__ffs(mask) - 1) && *reinterpret_cast<volatile int *>(flag) == 0)
+            atomicOr(flag, 1);
+        }
+        float deq[Q];
+        shifted_feq(m, deq);
+        if (!wait_phase_warp(c4, par, err)) break;
+        uint32_t v0[16], v1[16];
+        tmem_ld16(tm_row + TM_OUT, v0);
+        tmem_ld16(tm_row + TM_OUT + 16, v1);
+        tmem_wait_ld();
+        publish(m_o);
+        float o[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) o[i] = __uint_as_float(i < 16 ? v0[i] : v1[i - 16]);
+        project(o);
+        if (active) {
+          const float rw = m.rho * cp.omega;
+#pragma unroll
+          for (int i = 0; i < Q; ++i) d[i] = fmaf(cp.omega, deq[i] - d[i], d[i]) + rw * o[i];
+          const float Fx = cp.fx_y ? __ldg(cp.fx_y + P.y) : 0.f;
+          const float Fy = cp.fy_z ? __ldg(cp.fy_z + P.z) : 0.f;
+          const float Fz = cp.fz_x ? __ldg(cp.fz_x + P.x) : 0.f;
+          add_edm_force(m, Fx, Fy, Fz, d);
+          float *ob = out + (size_t)P.b * Q * vol + ((size_t)P.z * g.ny + P.y) * g.nx + P.x;
+#pragma unroll
+          for (int i = 0; i < Q; ++i) ob[(size_t)i * vol] = d[i];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        d[i] = dn[i];
+        dn[i] = df[i];
+      }
+      P = N;
+      N = F;
+      advance(F, g, st);
+    }
+  } else if (ok0) {
+    // ---------------- epilogues: WG0 the first, WG1 the second columns of each part
+    const int wg = warp >> 2;
+    const uint32_t tm_row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    const uint32_t m_1lo = map_cta(smem_u32(&S.b1lo), 0), m_1hi = map_cta(smem_u32(&S.b1hi), 0),
+                   m_2lo = map_cta(smem_u32(&S.b2lo), 0), m_2hi = map_cta(smem_u32(&S.b2hi), 0),
+                   m_3 = map_cta(smem_u32(&S.b3), 0);
+    const uint32_t c1a = smem_u32(&S.c1a), c1b = smem_u32(&S.c1b), c2a = smem_u32(&S.c2a), c2b = smem_u32(&S.c2b),
+                   c3 = smem_u32(&S.c3), c4 = smem_u32(&S.c4);
+    uint32_t par = 0;
+    bool ok = true;
+    for (int t = 0; t < count && ok; ++t, par ^= 1) {
+      // parts: lower and upper half of h1, of h2, then h3
+#pragma unroll 1
+      for (int e = 0; e < 5; ++e) {
+        // (the upper half of h1 takes columns that h3 of the previous tile held)
+        const uint32_t bar = e == 0 ? c1a : e == 1 ? c1b : e == 2 ? c2a : e == 3 ? c2b : c3;
+        if (!wait_phase_warp(bar, par, err) ||
+            (e == 1 && t > 0 && !wait_phase_warp(c4, par ^ 1, err))) {
+          ok = false;
+          break;
+        }
+        const int k0 = (e == 4 ? 4 : 5) * wg + (e & 1 ? 10 : 0);
+        const int steps = wg == 0 ? (e == 4 ? 4 : 5) : (e == 4 ? 3 : e & 1 ? 4 : 5);
+        const ColTable table = e < 2 ? col_h1() : e < 4 ? col_h2() : col_h3();
+        drain(tm_row, e < 4 ? TM_P : TM_A, table, k0, steps);
+        publish(e == 0 ? m_1lo : e == 1 ? m_1hi : e == 2 ? m_2lo : e == 3 ? m_2hi : m_3);
+      }
+    }
   }
 
-  // ---- teardown: every role has left its loop (normally or on an error)
+  // ---- teardown: every role of both CTAs has left its loop (normally or on an error)
+  __syncwarp();
   fence_before_sync();
-  __syncthreads();
+  cluster_sync();
   fence_after_sync();
-  if (warp == 0) tmem_dealloc(tmem, 512);
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   if (tid == 0 && S.err) atomicOr(timeout_flag, 1);
 }
 
-// FP32 packed weights -> BF16 operand tiles in the canonical K-major layout
-// (W1, W3, W4 whole; W2 as contiguous K chunks), biases in the constant-1 K
-// column, REPLICAS copies.
+// FP32 packed weights -> BF16 operand tiles in the canonical K-major layout,
+// biases in the constant-1 K column; one block of G_BYTES per CTA of a pair.
 __global__ void k3_prepare_weights(Mlp3 w, unsigned char *__restrict__ gw) {
   const int total = NH * KX + N4 * K4 + N3 * KH + NH * KH;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     float v = 0.f;
+    int rank;
     size_t off;
+    // rows of a hidden matrix: pass 0 | pass 1, each split between the CTAs
+    auto place_hidden = [&](int n, int k, int K, int base) {
+      const int hi = n >= NLO, m = hi ? n - NLO : n, half = hi ? R_HI : R_LO;
+      rank = m >= half;
+      off = base + (hi ? R_LO * K * 2 : 0) + canon_offset(m - rank * half, k, K);
+    };
+    // the row after a hidden layer's last unit yields the constant 1
+    auto one = [](bool here) { return here ? 1.f : 0.f; };
     if (e < NH * KX) {  // W1: rows n < 300, K 19 inputs, bias at k = 19
       const int n = e / KX, k = e % KX;
-      if (n < H1) v = k < Q ? w.w1[n * Q + k] : (k == Q ? w.b1[n] : 0.f);
-      off = G_W1 + canon_offset(n, k, KX);
+      v = n < H1 ? (k < Q ? w.w1[n * Q + k] : (k == Q ? w.b1[n] : 0.f)) : one(n == H1 && k == Q);
+      place_hidden(n, k, KX, G_W1);
     } else if (e < NH * KX + N4 * K4) {  // W4: rows n < 19, K 100, bias at k = 100
       const int f = e - NH * KX, n = f / K4, k = f % K4;
       if (n < Q) v = k < H3 ? w.w4[n * H3 + k] : (k == H3 ? w.b4[n] : 0.f);
-      off = G_W4 + canon_offset(n, k, K4);
+      rank = n >= N4 / 2;
+      off = G_W4 + canon_offset(n - rank * (N4 / 2), k, K4);
     } else if (e < NH * KX + N4 * K4 + N3 * KH) {  // W3: rows n < 100, K 300, bias at 300
       const int f = e - NH * KX - N4 * K4, n = f / KH, k = f % KH;
-      if (n < H3) v = k < H2 ? w.w3[n * H2 + k] : (k == H2 ? w.b3[n] : 0.f);
-      off = G_W3 + canon_offset(n, k, KH);
-    } else {  // W2 chunks
+      v = n < H3 ? (k < H2 ? w.w3[n * H2 + k] : (k == H2 ? w.b3[n] : 0.f)) : one(n == H3 && k == H2);
+      rank = n >= N3 / 2;
+      off = G_W3 + canon_offset(n - rank * (N3 / 2), k, KH);
+    } else {  // W2: rows n < 300, K 300, bias at 300
       const int f = e - NH * KX - N4 * K4 - N3 * KH, n = f / KH, k = f % KH;
-      if (n < H2) v = k < H1 ? w.w2[n * H1 + k] : (k == H1 ? w.b2[n] : 0.f);
-      const int c = k / KC;
-      off = G_W2 + (size_t)c * W2_CHUNK + canon_offset(n, k % KC, chunk_k(c));
+      v = n < H2 ? (k < H1 ? w.w2[n * H1 + k] : (k == H1 ? w.b2[n] : 0.f)) : one(n == H2 && k == H1);
+      place_hidden(n, k, KH, G_W2);
     }
-    const __nv_bfloat16 b = __float2bfloat16_rn(v);
-    for (int rep = 0; rep < REPLICAS; ++rep)
-      *reinterpret_cast<__nv_bfloat16 *>(gw + (size_t)rep * G_BYTES + off) = b;
+    *reinterpret_cast<__nv_bfloat16 *>(gw + (size_t)rank * G_BYTES + off) = __float2bfloat16_rn(v);
   }
 }
 
 }  // namespace
 
-size_t mlp_tc_weight_bytes() { return (size_t)G_BYTES * REPLICAS; }
+size_t mlp_tc_weight_bytes() { return 2 * (size_t)G_BYTES; }
 
 cudaError_t launch_prepare_weights_tc(const Mlp3 &w, void *gw, cudaStream_t s) {
   k3_prepare_weights<<<256, 256, 0, s>>>(w, static_cast<unsigned char *>(gw));
@@ -592,19 +646,28 @@ cudaError_t launch_prepare_weights_tc(const Mlp3 &w, void *gw, cudaStream_t s) {
 }
 
 cudaError_t launch_step_mlp_tc(const Grid3 &g, const float *in, float *out, const Collide3 &c,
-                               const void *gw, int sms, int *flag, int *timeout_flag,
+                               const void *gw, int sms, int *flag, int *timeout_flag, bool chain,
                                cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(k3_step_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((g.nx + 127) / 128) * g.ny * g.nz * g.batch;
-  if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const int grid = (int)(tiles < sms ? tiles : sms);
-  if (grid == 0) return cudaSuccess;
-  k3_step_mlp_tc<<<grid, THREADS, SMEM_BYTES, s>>>(in, out, g, c,
-                                                   static_cast<const unsigned char *>(gw), flag,
-                                                   timeout_flag);
-  return cudaGetLastError();
+  const long long pairs = ((long long)g.nodes() + 2 * TILE - 1) / (2 * TILE);
+  long long clusters = sms / 2;
+  if (clusters < 1) return cudaErrorInvalidConfiguration;
+  if (pairs < clusters) clusters = pairs;
+  if ((pairs + clusters - 1) / clusters > 0x7fffffffLL) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * clusters));
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k3_step_mlp_tc, in, out, g, c,
+                            static_cast<const unsigned char *>(gw), flag, timeout_flag);
 }
 
 }  // namespace d3

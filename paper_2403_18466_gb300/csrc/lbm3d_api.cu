@@ -183,7 +183,7 @@ int lbm3d_step(lbm3d_ctx *c, int n, lbm_collision kind, const lbm3d_weights *w) 
     float *out = c->buf[c->cur ^ 1];
     if (kind == LBM_MLP_BF16)
       CUDA_TRY(lbm::d3::launch_step_mlp_tc(c->g, in, out, c->cp, c->d_wtc, c->sms, c->d_flag,
-                                           c->d_flag + 1, c->stream));
+                                           c->d_flag + 1, s > 0, c->stream));
     else if (kind == LBM_MLP_F32)
       CUDA_TRY(lbm::d3::launch_step_mlp_f32(c->g, in, out, c->cp, c->d_wf32, c->d_flag,
                                             c->stream));

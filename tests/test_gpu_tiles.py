@@ -10,7 +10,7 @@ import pytest
 
 import oracle.d3q19 as o3
 from paper_2403_18466_gb300 import inputs
-from test_gpu_d3q19 import W, _dev, _np, _weights, field3d, lbm, wpe  # noqa: F401
+from test_gpu_d3q19 import _dev, _np, _weights, emulate_tc_step, field3d, lbm, wpe  # noqa: F401
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -34,3 +34,42 @@ def test_d3q19_f32_tiles(lbm, nx, ny, nz, B):  # noqa: F811
     got = _np(lat.get_state())
     assert wpe(got, ref) <= 1e-5 and wpe(ref, bgk) > 100 * wpe(got, ref)
     assert lat.status() == lbm.LBM_OK
+
+
+@pytest.mark.parametrize("nx,ny,nz,B", [(127, 1, 1, 1), (43, 3, 1, 1), (16, 16, 1, 1),
+                                        (257, 1, 1, 1), (5, 17, 3, 3), (2, 1, 129, 2)])
+def test_d3q19_tc_tile_pairs(lbm, nx, ny, nz, B):  # noqa: F811
+    """Tensor-core learned D3Q19 step (pairs of 128-node tiles): within 5e-3 of
+    the learned correction of the bf16-rounding restatement, as on whole rows."""
+    tau, F, m = 0.6, 2e-4, 1
+    theta = _weights(24, out_scale=0.01)
+    f = field3d(B, nz, ny, nx, seed=51, neq=0.02)
+    lat = lbm.Lattice3D(nx, ny, nz, B, tau=tau, force_amp=F, force_mode=m, device=DEV)
+    lat.set_state(_dev(f))
+    g = o3.stream_push(_np(lat.get_state()))
+    th = torch.tensor(theta, dtype=torch.float32, device=DEV)
+    lat.step(1, "mlp_bf16", lbm.weights3d_struct(th))
+    got = _np(lat.get_state())
+    ref = emulate_tc_step(g, theta, tau, F, m)
+    bgk = o3.stream_pull(o3.step(o3.BGK, g, o3.params(tau, force_amp=F, force_mode=m)))
+    corr = wpe(ref, bgk)
+    assert wpe(got, ref) <= 5e-3 * corr and corr > 1e-3
+    assert lat.status() == lbm.LBM_OK
+
+
+def test_d3q19_tc_many_tiles(lbm):  # noqa: F811
+    """Every CTA pair walks several tile pairs that span rows and planes: a
+    lattice repeated 5 x 5 along x and y evolves as copies of itself, so each
+    copy, whatever tiles it falls into, has the bits of the single lattice."""
+    nx, ny, nz, r = 60, 26, 2, 5
+    f = _dev(field3d(1, nz, ny, nx, seed=52, neq=0.02))
+    w = lbm.weights3d_struct(torch.tensor(_weights(25, out_scale=0.0005), dtype=torch.float32,
+                                          device=DEV))
+    small = lbm.Lattice3D(nx, ny, nz, 1, tau=0.6, device=DEV)
+    large = lbm.Lattice3D(nx * r, ny * r, nz, 1, tau=0.6, device=DEV)
+    small.set_state(f)
+    large.set_state(f.repeat(1, 1, 1, r, r).contiguous())
+    for lat in (small, large):
+        lat.step(3, "mlp_bf16", w)
+        assert lat.status() == lbm.LBM_OK
+    assert torch.equal(large.get_state(), small.get_state().repeat(1, 1, 1, r, r))
