@@ -28,10 +28,16 @@ struct MlpF32 {
 };
 
 // step_fp32.cu ---------------------------------------------------------------
-cudaError_t launch_step_bgk(const Grid &g, const float *in, float *out, const CollideParams &p,
-                            int *flag, cudaStream_t s);
-cudaError_t launch_step_smag(const Grid &g, const float *in, float *out, const CollideParams &p,
-                             int *flag, cudaStream_t s);
+// Plain collisions: a launch advances t steps, 1 <= t <= step_plan(g).steps;
+// tile: side of the small-lattice kernel's tiles, 0 for the others.
+struct StepPlan {
+  int steps, tile;
+};
+StepPlan step_plan(const Grid &g);
+cudaError_t launch_steps_bgk(const Grid &g, const float *in, float *out, const CollideParams &p,
+                             int t, int *flag, cudaStream_t s);
+cudaError_t launch_steps_smag(const Grid &g, const float *in, float *out, const CollideParams &p,
+                              int t, int *flag, cudaStream_t s);
 cudaError_t launch_set_state(const Grid &g, const float *f_pre, float *state, cudaStream_t s);
 cudaError_t launch_get_state(const Grid &g, const float *state, float *f_pre, cudaStream_t s);
 cudaError_t launch_init_equilibrium(const Grid &g, const float *rho, const float *ux,

@@ -89,15 +89,18 @@ MlpF32 f32_view(const lbm_weights *w) {
   return m;
 }
 
-// One step from `in` to `out` with the given collision.  `chain`: the previous
+// One launch from `in` to `out` with the given collision: `steps` steps of a
+// plain collision (at most lbm::step_plan's), one of a learned one.  `chain`: the previous
 // operation on the stream is a step of the same collision issued by the same
 // call (no copy or other kernel in between), so the tensor-core step may start
 // its prologue while that one finishes (programmatic dependent launch).
 cudaError_t one_step(lbm_ctx *c, const float *in, float *out, lbm_collision kind,
-                     const lbm_weights *w, bool chain = false) {
+                     const lbm_weights *w, bool chain = false, int steps = 1) {
   switch (kind) {
-    case LBM_BGK: return lbm::launch_step_bgk(c->g, in, out, c->cp, c->d_flag, c->stream);
-    case LBM_SMAG: return lbm::launch_step_smag(c->g, in, out, c->cp, c->d_flag, c->stream);
+    case LBM_BGK:
+      return lbm::launch_steps_bgk(c->g, in, out, c->cp, steps, c->d_flag, c->stream);
+    case LBM_SMAG:
+      return lbm::launch_steps_smag(c->g, in, out, c->cp, steps, c->d_flag, c->stream);
     case LBM_MLP_F32:
       return lbm::launch_step_mlp_f32(c->g, in, out, c->cp, f32_view(w), c->d_flag, c->stream);
     case LBM_MLP_BF16: {
@@ -250,8 +253,15 @@ int lbm_step(lbm_ctx *c, int n, lbm_collision kind, const lbm_weights *w) {
   if (kind < LBM_BGK || kind > LBM_MLP_F32) return LBM_ERR_ARG;
   const int wc = check_weights(kind, w);
   if (wc != LBM_OK) return wc;
-  for (int s = 0; s < n; ++s) {
-    CUDA_TRY(one_step(c, c->buf[c->cur], c->buf[c->cur ^ 1], kind, w, s > 0));
+  // Launches: as few as the steps per launch allow, but of the parity of n, so
+  // that the state ends in the same buffer as after n single steps (a captured
+  // sequence of an even number of steps can then be replayed on its result).
+  const int most = kind <= LBM_SMAG ? lbm::step_plan(c->g).steps : 1;
+  int launches = n / most + (n % most ? 1 : 0);
+  if ((n - launches) & 1) ++launches;
+  for (int s = 0; s < launches; ++s) {
+    const int steps = n / launches + (s < n % launches ? 1 : 0);
+    CUDA_TRY(one_step(c, c->buf[c->cur], c->buf[c->cur ^ 1], kind, w, s > 0, steps));
     c->cur ^= 1;
   }
   return LBM_OK;

@@ -9,7 +9,9 @@
 // stores into the next buffer at x.  Algorithmic traffic: 36 B read + 36 B
 // written per node (FP32 D2Q9).
 //
-// Fast path (nx % 4 == 0): one thread owns 4 consecutive nodes of a row.
+// Several steps of one call run as one launch (k_steps_tile; k_steps_small on
+// small lattices).  Single steps:
+// nx % 4 == 0: one thread owns 4 consecutive nodes of a row.
 // Every plane row is read with aligned 128-bit loads; the one value that a
 // shifted plane (c_x = +-1) needs from the neighbouring 4-node group comes
 // from the adjacent lane by a warp shuffle, and only the warp's edge lanes
@@ -29,8 +31,25 @@ constexpr int SCALAR_THREADS = 128;
 
 enum { KIND_BGK = 0, KIND_SMAG = 1 };
 
-// Collide one node in place (shifted representation), add the force.
-// Returns true if the node is unstable (|u| >= 0.4 or not finite).
+// Pi^neq : Pi^neq with Pi^neq_ab = sum_i c_ia c_ib n_i, n = f - feq (SI sec. 1).
+template <class T>
+__device__ __forceinline__ T stress_norm(const T n[Q]) {
+  const T dg = v_add(v_add(n[5], n[6]), v_add(n[7], n[8]));
+  const T pxx = v_add(v_add(n[1], n[3]), dg), pyy = v_add(v_add(n[2], n[4]), dg);
+  const T pxy = v_add(v_sub(n[5], n[6]), v_sub(n[7], n[8]));
+  return v_fma(pyy, pyy, v_fma(v_mul(v_c<T>(2.0f), pxy), pxy, v_mul(pxx, pxx)));
+}
+__device__ __forceinline__ float smag_omega(float pp, float inv_rho, const CollideParams &p) {
+  return smagorinsky_omega(pp, inv_rho, p.tau, p.tau0_sq, p.smag_c18);
+}
+__device__ __forceinline__ float2 smag_omega(float2 pp, float2 inv_rho, const CollideParams &p) {
+  return make_float2(smag_omega(pp.x, inv_rho.x, p), smag_omega(pp.y, inv_rho.y, p));
+}
+
+// Collide one node (float) or two (float2: packed f32x2, half the issue slots)
+// in place (shifted representation), add the force.  Every operation is
+// rounded explicitly, so both forms, and every kernel that uses them, give the
+// same bits.  Returns true if a node is unstable (|u| >= 0.4 or not finite).
 template <int KIND>
 __device__ __forceinline__ bool collide_node(float d[Q], const CollideParams &p, float fx) {
   const Moments m = node_moments(d);
@@ -39,22 +58,35 @@ __device__ __forceinline__ bool collide_node(float d[Q], const CollideParams &p,
   shifted_feq(m, deq);
   float omega = p.omega;
   if (KIND == KIND_SMAG) {
-    // Pi^neq_ab = sum_i c_ia c_ib (f_i - feq_i); tau_eff closed form (SI sec. 1)
     float n[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) n[i] = d[i] - deq[i];
-    const float pxx = (n[1] + n[3]) + ((n[5] + n[6]) + (n[7] + n[8]));
-    const float pyy = (n[2] + n[4]) + ((n[5] + n[6]) + (n[7] + n[8]));
-    const float pxy = (n[5] - n[6]) + (n[7] - n[8]);
-    omega = smagorinsky_omega(pxx * pxx + 2.0f * pxy * pxy + pyy * pyy, m.inv_rho, p.tau,
-                              p.tau0_sq, p.smag_c18);
+    for (int i = 0; i < Q; ++i) n[i] = v_sub(d[i], deq[i]);
+    omega = smag_omega(stress_norm(n), m.inv_rho, p);
   }
 #pragma unroll
   for (int i = 0; i < Q; ++i) d[i] = bgk_relax(d[i], deq[i], omega);
   add_edm_force_x(m, fx, d);  // fx = 0 without forcing
   return bad;
 }
-
+template <int KIND>
+__device__ __forceinline__ bool collide_node(float2 d[Q], const CollideParams &p, float2 fx,
+                                             bool act_x, bool act_y) {
+  const MomentsT<float2> m = node_moments(d);
+  const bool bad = is_unstable(m, act_x, act_y);
+  float2 deq[Q];
+  shifted_feq(m, deq);
+  float2 omega = make_float2(p.omega, p.omega);
+  if (KIND == KIND_SMAG) {
+    float2 n[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) n[i] = v_sub(d[i], deq[i]);
+    omega = smag_omega(stress_norm(n), m.inv_rho, p);
+  }
+#pragma unroll
+  for (int i = 0; i < Q; ++i) d[i] = bgk_relax(d[i], deq[i], omega);
+  add_edm_force_x(m, fx, d);
+  return bad;
+}
 __device__ __forceinline__ float4 ldg4(const float *p) {
   return __ldg(reinterpret_cast<const float4 *>(p));
 }
@@ -163,23 +195,225 @@ __global__ void __launch_bounds__(SCALAR_THREADS)
   for (int i = 0; i < Q; ++i) ob[i * plane + (size_t)y * nx + x] = d[i];
 }
 
+// Several steps in one pass over memory: a block advances a tile by t steps
+// (t <= MT_MOST), the first on a region of MT_X x MT_Y nodes and each later one
+// on a ring less, and stores the (MT_X - 2 (t - 1)) x (MT_Y - 2 (t - 1)) nodes
+// that are then complete, so the state crosses HBM (or L2) once per t steps.
+// A thread owns MT_PP pairs of adjacent rows of one column: the two nodes of a
+// pair run in packed f32x2 arithmetic, and their 18 populations are plain
+// 32-bit loads (a warp reads 32 adjacent columns of a row), with no shuffles
+// and no moves to form the pairs.  Between steps the post-collision
+// populations are in shared memory, replaced in place.
+// What bounds it: the FP32 pipe and instruction issue (64 % of the slots at
+// 1024^2 Smagorinsky, ~190 instructions per computed node), no longer HBM; t = 3
+// on a 64 x 16 region recomputes 21 % of the nodes.  Measured (GB300, us per
+// step, BGK / Smagorinsky, one step per launch before):
+//   256^2   3.2 / 3.6 -> 1.6 / 1.9       512^2   4.6 / 5.0 -> 2.9 / 3.5
+//   1024^2 10.0 / 10.6 -> 8.4 / 10.4    2048^2  49.5 / 51.8 -> 30.2 / 36.6
+//   4096^2  185 / 189 -> 116 / 140      1001^2  11.0 / 12.0 -> 8.1 / 9.6
+// t = 2 or 4, 32- or 24-row regions and other block sizes were within 15 % or
+// slower; four nodes per thread with 128-bit loads and shuffles (t = 2) reached
+// 41 us at 2048^2, the same with the next tile's cp.async copies in flight 44.
+constexpr int MT_X = 64, MT_THREADS = 256, MT_PR = MT_THREADS / MT_X;
+constexpr int MT_PP = 2;               // pairs of rows per thread
+constexpr int MT_Y = 2 * MT_PR * MT_PP;  // rows of the region
+constexpr int MT_MOST = 3;
+
+template <int KIND>
+__global__ void __launch_bounds__(MT_THREADS, 3)
+    k_steps_tile(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int t,
+                 CollideParams p, int *flag) {
+  constexpr int RY = MT_Y, PP = MT_PP;
+  extern __shared__ float tile[];  // [Q][RY][MT_X]
+  umma::griddep_wait();  // launched as a dependent of the previous step
+  umma::griddep_launch_dependents();
+  const int lx = threadIdx.x % MT_X, pr = threadIdx.x / MT_X;
+  const int X0 = (int)blockIdx.x * (MT_X - 2 * (t - 1)) - (t - 1);
+  const int Y0 = (int)blockIdx.y * (RY - 2 * (t - 1)) - (t - 1);
+  const size_t plane = (size_t)nx * ny;
+  auto wrap = [](int a, int n) { return a < 0 ? (a % n + n) % n : (a >= n ? a % n : a); };
+  bool bad = false;
+  float2 d[PP][Q];
+  float2 fx[PP];
+  {
+    // step 1, from global memory
+    const float *gb = in + (size_t)blockIdx.z * Q * plane;
+    const uint32_t x = wrap(X0 + lx, nx), X = nx;
+    // x - c_x at 1 + c_x
+    const uint32_t xs[3] = {x == X - 1 ? 0 : x + 1, x, x == 0 ? X - 1 : x - 1};
+#pragma unroll
+    for (int j = 0; j < PP; ++j) {
+      const int y0 = wrap(Y0 + 2 * (pr + MT_PR * j), ny);
+      const int y1 = y0 == ny - 1 ? 0 : y0 + 1;
+      const int ym = y0 == 0 ? ny - 1 : y0 - 1, yp = y1 == ny - 1 ? 0 : y1 + 1;
+      // source rows of the two nodes, y - c_y at 1 + c_y
+      const uint32_t r0[3] = {y1 * X, y0 * X, ym * X}, r1[3] = {yp * X, y1 * X, y0 * X};
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const float *pl = gb + i * plane;
+        d[j][i] = make_float2(__ldg(pl + (r0[1 + cy(i)] + xs[1 + cx(i)])),
+                              __ldg(pl + (r1[1 + cy(i)] + xs[1 + cx(i)])));
+      }
+      fx[j] = p.force ? make_float2(__ldg(p.force + y0), __ldg(p.force + y1))
+                      : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int j = 0; j < PP; ++j) bad |= collide_node<KIND>(d[j], p, fx[j], true, true);
+  }
+#pragma unroll 1
+  for (int s = 1; s < t; ++s) {
+    if (s > 1) __syncthreads();  // the previous state is read
+#pragma unroll
+    for (int j = 0; j < PP; ++j) {
+      float *o = tile + 2 * (pr + MT_PR * j) * MT_X + lx;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        o[i * RY * MT_X] = d[j][i].x;
+        o[i * RY * MT_X + MT_X] = d[j][i].y;
+      }
+    }
+    __syncthreads();
+    // nodes at least s from the region's edge; the other node of a pair that
+    // straddles the limit reads a clamped row and is not used
+    if (lx >= s && lx < MT_X - s) {
+#pragma unroll
+      for (int j = 0; j < PP; ++j) {
+        const int r = 2 * (pr + MT_PR * j);
+        if (r + 1 < s || r >= RY - s) continue;
+        const int rm = r == 0 ? 0 : r - 1, rp = r + 2 == RY ? r + 1 : r + 2;
+        const int a[3] = {r + 1, r, rm}, b[3] = {rp, r + 1, r};
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const float *pl = tile + i * RY * MT_X + lx - cx(i);
+          d[j][i] = make_float2(pl[a[1 + cy(i)] * MT_X], pl[b[1 + cy(i)] * MT_X]);
+        }
+        bad |= collide_node<KIND>(d[j], p, fx[j], r >= s, r + 1 < RY - s);
+      }
+    }
+  }
+  flag_unstable(bad, flag);
+  const int e = t - 1, x = X0 + lx;
+  if (lx < e || lx >= MT_X - e || x >= nx) return;
+  float *ob = out + (size_t)blockIdx.z * Q * plane;
+#pragma unroll
+  for (int j = 0; j < PP; ++j) {
+    const int r = 2 * (pr + MT_PR * j), y = Y0 + r;
+    const uint32_t at = (uint32_t)y * (uint32_t)nx + (uint32_t)x;
+    if (r >= e && r < RY - e && y < ny)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) (ob + i * plane)[at] = d[j][i].x;
+    if (r + 1 >= e && r + 1 < RY - e && y + 1 < ny)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) (ob + i * plane)[at + (uint32_t)nx] = d[j][i].y;
+  }
+}
+
+// Several steps in one launch for small lattices, where the launches
+// are the cost (64^2: 2.9 us per step with one step per launch, 0.66 with 8): a block advances a tile of ts x ts nodes by t steps, the first
+// on the tile and the t - 1 nodes around it (one node per thread), each later
+// one on a ring less, between two shared-memory buffers.
+constexpr int MS_SIDE = 22;               // ts + 2 (t - 1) at most
+constexpr int MS_NODES = MS_SIDE * MS_SIDE;
+constexpr int MS_THREADS = 512;
+static_assert(MS_NODES <= MS_THREADS, "one node per thread");
+
+template <int KIND>
+__global__ void __launch_bounds__(MS_THREADS, 2)
+    k_steps_small(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int ts,
+                  int t, CollideParams p, int *flag) {
+  extern __shared__ float buf[];  // [2][Q][MS_NODES]
+  umma::griddep_wait();           // launched as a dependent of the previous step
+  umma::griddep_launch_dependents();
+  const int side = ts + 2 * (t - 1);
+  const int ly = threadIdx.x / side, lx = threadIdx.x - ly * side;
+  const size_t plane = (size_t)nx * ny;
+  const bool node = ly < side;
+  int x = 0, y = 0;
+  if (node) {
+    x = ((int)blockIdx.x * ts - (t - 1) + lx) % nx;
+    y = ((int)blockIdx.y * ts - (t - 1) + ly) % ny;
+    x = x < 0 ? x + nx : x;
+    y = y < 0 ? y + ny : y;
+  }
+  const float fx = p.force && node ? __ldg(p.force + y) : 0.0f;
+  // this node takes part in the first `steps` steps
+  const int edge = min(min(lx, side - 1 - lx), min(ly, side - 1 - ly));
+  const int steps = node ? min(edge + 1, t) : 0;
+  float d[Q];
+  bool bad = false;
+  if (node) {
+    pull_node(in + (size_t)blockIdx.z * Q * plane, plane, nx, ny, x, y, d);
+    bad = collide_node<KIND>(d, p, fx);
+  }
+  for (int s = 1; s < t; ++s) {
+    float *b = buf + (s & 1) * (Q * MS_NODES);
+    if (s <= steps)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) b[i * MS_NODES + threadIdx.x] = d[i];
+    __syncthreads();
+    if (s < steps) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) d[i] = b[i * MS_NODES + (int)threadIdx.x - cy(i) * side - cx(i)];
+      bad |= collide_node<KIND>(d, p, fx);
+    }
+  }
+  flag_unstable(bad, flag);
+  const int gx = blockIdx.x * ts + lx - (t - 1), gy = blockIdx.y * ts + ly - (t - 1);
+  if (steps == t && gx < nx && gy < ny) {
+    float *ob = out + (size_t)blockIdx.z * Q * plane + (size_t)gy * nx + gx;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) ob[i * plane] = d[i];
+  }
+}
+
 // Programmatic dependent launch: the kernel waits for the previous kernel on
 // the stream before its first global access, so its CTAs may be scheduled
 // while that kernel's last CTAs finish (it hides the launch gap between steps).
 template <int KIND>
-cudaError_t launch_step(const Grid &g, const float *in, float *out, const CollideParams &p,
-                        int *flag, cudaStream_t s) {
-  const bool vec = g.nx % 4 == 0;
+cudaError_t launch_steps(const Grid &g, const float *in, float *out, const CollideParams &p, int t,
+                         int *flag, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = vec ? dim3((g.nx / 4 + VEC_THREADS - 1) / VEC_THREADS, g.ny, g.batch)
-                    : dim3((g.nx + SCALAR_THREADS - 1) / SCALAR_THREADS, g.ny, g.batch);
-  cfg.blockDim = dim3(vec ? VEC_THREADS : SCALAR_THREADS);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const StepPlan plan = step_plan(g);
+  if (t > 1 && plan.tile > 0) {
+    static bool attr_done = false;
+    const int smem = 2 * Q * MS_NODES * (int)sizeof(float);
+    if (!attr_done) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          k_steps_small<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e != cudaSuccess) return e;
+      attr_done = true;
+    }
+    cfg.gridDim = dim3((g.nx + plan.tile - 1) / plan.tile, (g.ny + plan.tile - 1) / plan.tile,
+                       g.batch);
+    cfg.blockDim = dim3(MS_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    return cudaLaunchKernelEx(&cfg, k_steps_small<KIND>, in, out, g.nx, g.ny, plan.tile, t, p, flag);
+  }
+  if (t > 1) {
+    static bool attr_done = false;
+    const int smem = Q * MT_Y * MT_X * (int)sizeof(float);
+    if (!attr_done) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          k_steps_tile<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e != cudaSuccess) return e;
+      attr_done = true;
+    }
+    const int tw = MT_X - 2 * (t - 1), th = MT_Y - 2 * (t - 1);
+    cfg.gridDim = dim3((g.nx + tw - 1) / tw, (g.ny + th - 1) / th, g.batch);
+    cfg.blockDim = dim3(MT_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    return cudaLaunchKernelEx(&cfg, k_steps_tile<KIND>, in, out, g.nx, g.ny, t, p, flag);
+  }
+  const bool vec = g.nx % 4 == 0;
+  cfg.gridDim = vec ? dim3((g.nx / 4 + VEC_THREADS - 1) / VEC_THREADS, g.ny, g.batch)
+                    : dim3((g.nx + SCALAR_THREADS - 1) / SCALAR_THREADS, g.ny, g.batch);
+  cfg.blockDim = dim3(vec ? VEC_THREADS : SCALAR_THREADS);
   if (vec) return cudaLaunchKernelEx(&cfg, k_step_vec<KIND>, in, out, g.nx, g.ny, p, flag);
   return cudaLaunchKernelEx(&cfg, k_step_scalar<KIND>, in, out, g.nx, g.ny, p, flag);
 }
@@ -473,14 +707,25 @@ __global__ void k_shift(const float *__restrict__ in, float *__restrict__ out, i
 
 }  // namespace
 
-cudaError_t launch_step_bgk(const Grid &g, const float *in, float *out, const CollideParams &p,
-                            int *flag, cudaStream_t s) {
-  return launch_step<KIND_BGK>(g, in, out, p, flag, s);
+// Up to 128^2 nodes a step is shorter than its launch: 8 steps per launch on
+// 8 x 8 tiles, mostly recomputed rings, take 0.7 us per step at 64^2 and 1.2 at
+// 128^2 (the tile kernel 1.4 and 1.4, one step per launch 3.0 and 2.7); at 256^2
+// they take 2.6 us against 1.6.  Planes of 2^31 nodes or more (beyond the tile
+// kernel's 32-bit offsets) go step by step.
+StepPlan step_plan(const Grid &g) {
+  if (g.nodes() <= 128 * 128) return {8, 8};
+  if (g.plane() < 1u << 31) return {MT_MOST, 0};
+  return {1, 0};
 }
 
-cudaError_t launch_step_smag(const Grid &g, const float *in, float *out, const CollideParams &p,
-                             int *flag, cudaStream_t s) {
-  return launch_step<KIND_SMAG>(g, in, out, p, flag, s);
+cudaError_t launch_steps_bgk(const Grid &g, const float *in, float *out, const CollideParams &p,
+                             int t, int *flag, cudaStream_t s) {
+  return launch_steps<KIND_BGK>(g, in, out, p, t, flag, s);
+}
+
+cudaError_t launch_steps_smag(const Grid &g, const float *in, float *out, const CollideParams &p,
+                              int t, int *flag, cudaStream_t s) {
+  return launch_steps<KIND_SMAG>(g, in, out, p, t, flag, s);
 }
 
 cudaError_t launch_set_state(const Grid &g, const float *f_pre, float *state, cudaStream_t s) {

@@ -73,3 +73,33 @@ def test_d3q19_tc_many_tiles(lbm):  # noqa: F811
         lat.step(3, "mlp_bf16", w)
         assert lat.status() == lbm.LBM_OK
     assert torch.equal(large.get_state(), small.get_state().repeat(1, 1, 1, r, r))
+
+
+@pytest.mark.parametrize("kind", ["bgk", "smag"])
+@pytest.mark.parametrize("nx,ny,B", [(1, 1, 1), (3, 5, 2), (9, 8, 1), (64, 64, 1), (128, 128, 1),
+                                     (129, 128, 1), (61, 300, 1), (16, 1100, 1), (1100, 15, 2),
+                                     (181, 97, 3)])
+@pytest.mark.parametrize("n", [2, 3, 4, 7, 16, 17])
+def test_several_steps_per_launch(lbm, kind, nx, ny, B, n):  # noqa: F811
+    """n steps of one call (several steps per launch, recomputed rings around the
+    tiles) have the bits of n calls of one step, end in the same buffer, and
+    flag an unstable node alike."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(nx + 7 * ny + n)
+    rnd = lambda: torch.rand((B, ny, nx), generator=g, device=DEV) - 0.5
+    rho, ux, uy = 1 + 0.02 * rnd(), 0.1 * rnd(), 0.1 * rnd()
+    args = dict(tau=0.53, smag_cs=0.2, force_amp=1e-4, force_mode=1, device=DEV)
+    one, many = lbm.Lattice(nx, ny, B, **args), lbm.Lattice(nx, ny, B, **args)
+    for fast in (False, True):
+        if fast:  # one node beyond the stability limit
+            ux[-1, -1, -1] = 0.45
+        for lat in (one, many):
+            lat.clear_status()
+            lat.init_equilibrium(rho, ux, uy)
+        for _ in range(n):
+            one.step(1, kind)
+        many.step(n, kind)
+        assert torch.equal(one.get_state(), many.get_state())
+        assert (one.state_buffer() == one.bufs[0].data_ptr()) == \
+            (many.state_buffer() == many.bufs[0].data_ptr())
+        assert one.status() == many.status() == (lbm.LBM_ERR_UNSTABLE if fast else lbm.LBM_OK)
