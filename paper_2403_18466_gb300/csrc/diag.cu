@@ -4,12 +4,11 @@
 //
 // Structure functions: S^p(r) = < [(u(x + r e) - u(x)) . e]^p >, p = 1..6,
 // r = 1..rmax, averaged over every node and the two lattice directions
-// e = x^, y^ (periodic).  For rmax <= 256: row segments and column strips of
-// the field staged in shared memory with an rmax halo, one thread per
-// separation; otherwise one block per (r, chunk of rows).  Either way
-// per-thread FP32 sums over at most 32 nodes are flushed into FP64
-// accumulators and per-block partials are added in a fixed order, so results
-// are reproducible.
+// e = x^, y^ (periodic).  For rmax <= 256: strips of 32 lines staged in shared
+// memory with an rmax halo, one thread per separation; otherwise one block per
+// (r, chunk of rows).  Either way per-thread FP32 sums over at most 32 nodes are
+// flushed into FP64 (or FP32-pair) accumulators and per-block FP64 partials are
+// added in a fixed order, so results are reproducible.
 //
 // Energy spectrum: E(k) = 1/2 sum_{round(|k'|) = k} |u_hat(k')|^2 / N^2 for the
 // unnormalised 2D DFT (N = nx ny), averaged over the batch, so that the sum
@@ -83,129 +82,202 @@ __global__ void __launch_bounds__(SF_THREADS)
 }
 
 // Tiled form for rmax <= SFT_R (the usual case): one pass over the field per
-// direction instead of one per separation.  Thread r - 1 of a block owns
-// separation r; the block stages a periodic segment of the field with an rmax
-// halo in shared memory, and for every node of it thread r takes
-// s[x + r] - s[x] (the first read is a broadcast, the second conflict-free).
-// Each thread sums at most 32 terms in FP32 before adding them to its FP64
-// sums; each block writes its 6 sums per separation; a last kernel adds the
-// blocks in a fixed order.
-constexpr int SFT_R = 256;   // separations per block (threads)
-constexpr int SFT_X = 1024;  // nodes of a row segment (x direction)
-constexpr int SFT_RB = 16;   // rows per x block
-constexpr int SFT_C = 32;    // columns of a y strip
-constexpr int SFT_Y = 256;   // rows of a y strip
-constexpr int SFT_CS = SFT_C + 1;  // padded column stride
+// direction instead of one per separation.  A block stages 32 rows (for the x
+// increments) or 32 columns (y) over h positions along the increments and the
+// next rmax ones (periodic) in shared memory; thread r - 1 owns separation r.
+// Two nodes at a time in packed f32x2: two rows for the x increments, stored as
+// [x][row] so that 16-byte loads give four rows (a stride of 36 floats keeps
+// them free of bank conflicts); two positions for the y increments, stored as
+// [column][y].  Nine FMA-pipe operations per increment for its six powers
+// bound the kernel.  Each lane sums 32 terms, adjacent in x, in FP32 (S^1 is the
+// rounding left of a sum that cancels, so the order is part of the result)
+// before they go into its running sum, a pair of FP32 numbers kept by
+// error-free additions (about 48 bits): FP64 additions, at 1/64 of the FP32
+// rate, took as long as all the rest.
+constexpr int SFT_R = 256;    // largest separation
+constexpr int SF_LINES = 32;
+constexpr int SF_STRIDE = SF_LINES + 4;  // of a position of the x increments
+constexpr int SF_MOST_BLOCKS = 4096;
 
-struct SfAcc {
-  double acc[6];
-  float facc[6];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      acc[p] = 0.0;
-      facc[p] = 0.f;
-    }
-  }
-  __device__ __forceinline__ void add(float d) {
-    const float d2 = d * d, d3 = d2 * d, d4 = d2 * d2;
-    facc[0] += d;
-    facc[1] += d2;
-    facc[2] += d3;
-    facc[3] += d4;
-    facc[4] += d4 * d;
-    facc[5] += d3 * d3;
-  }
-  __device__ __forceinline__ void flush() {
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      acc[p] += (double)facc[p];
-      facc[p] = 0.f;
-    }
-  }
+// (hi, lo) += f without rounding error but in lo (Knuth's two-sum)
+__device__ __forceinline__ void pair_add(float2 &hi, float2 &lo, float2 f) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 s = __fadd2_rn(hi, f);
+  const float2 b = __ffma2_rn(hi, m1, s);
+  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(b, m1, s), m1, hi), __ffma2_rn(b, m1, f));
+  lo = __fadd2_rn(lo, e);
+  hi = s;
+}
+
+struct SfShape {
+  int h;             // positions per block
+  int bx, by;        // blocks of the x and of the y increments
+  int segs_x, segs_y;  // blocks along the axis
 };
 
 __global__ void __launch_bounds__(SFT_R)
-    k_sf_rows(const float *__restrict__ ux, int nx, int rows, int rmax, double *__restrict__ part) {
-  extern __shared__ float seg[];  // SFT_X + rmax
-  const int x0 = blockIdx.x * SFT_X;
-  const int w = min(SFT_X, nx - x0);
-  const int row0 = blockIdx.y * SFT_RB, row1 = min(row0 + SFT_RB, rows);
-  const int r = threadIdx.x + 1;
-  SfAcc a;
-  a.zero();
-  for (int row = row0; row < row1; ++row) {
-    const float *u = ux + (size_t)row * nx;  // row b ny + y of the [B][ny][nx] field
-    __syncthreads();
-    for (int i = threadIdx.x; i < w + rmax; i += SFT_R) seg[i] = u[(x0 + i) % nx];
-    __syncthreads();
-    if (r <= rmax) {
-      for (int xb = 0; xb < w; xb += 32) {
-        const int xe = min(xb + 32, w);
-        for (int x = xb; x < xe; ++x) a.add(seg[x + r] - seg[x]);
-        a.flush();
+    k_sf_strips(const float *__restrict__ ux, const float *__restrict__ uy, int nx, int ny,
+                int batch, int rmax, SfShape sh, double *__restrict__ part) {
+  extern __shared__ __align__(16) float strip[];  // (h + rmax) positions of 32 lines
+  const bool along_x = (int)blockIdx.x < sh.bx;
+  const int ystride = (sh.h + rmax + 2) / 2 * 2 + 1;  // odd: a warp stages 32 columns
+  const int rt = (rmax + 31) / 32 * 32;  // threads per slice; slices share the positions
+  const int slices = blockDim.x / rt, slice = threadIdx.x / rt, r = threadIdx.x % rt + 1;
+  int h;
+  if (along_x) {
+    // 32 rows of the flattened batch, positions along x
+    const int p0 = blockIdx.x % sh.segs_x * sh.h, l0 = blockIdx.x / sh.segs_x * SF_LINES;
+    h = min(sh.h, nx - p0);
+    const int lw = min(SF_LINES, ny * batch - l0);
+    for (int l = threadIdx.x / 32; l < SF_LINES; l += blockDim.x / 32)
+      for (int j = threadIdx.x % 32; j < h + rmax; j += 32)
+        strip[j * SF_STRIDE + l] = l < lw ? ux[(size_t)(l0 + l) * nx + (p0 + j) % nx] : 0.f;
+  } else {
+    // 32 columns of one lattice, positions along y
+    const int blk = blockIdx.x - sh.bx, strips = (nx + SF_LINES - 1) / SF_LINES;
+    const int l0 = blk % strips * SF_LINES, q = blk / strips;
+    const int p0 = q % sh.segs_y * sh.h;
+    h = min(sh.h, ny - p0);
+    const int lw = min(SF_LINES, nx - l0), l = threadIdx.x % 32;
+    const float *u = uy + (size_t)(q / sh.segs_y) * nx * ny + l0 + l;
+    for (int j = threadIdx.x / 32; j < h + rmax; j += blockDim.x / 32)
+      strip[l * ystride + j] = l < lw ? u[(size_t)((p0 + j) % ny) * nx] : 0.f;
+  }
+  __syncthreads();
+  float2 hi[6], lo[6];
+#pragma unroll
+  for (int p = 0; p < 6; ++p) hi[p] = lo[p] = make_float2(0.f, 0.f);
+  const float2 m1 = make_float2(-1.f, -1.f);
+  auto add = [](float2 (&f)[6], float2 d) {
+    const float2 d2 = __fmul2_rn(d, d), d3 = __fmul2_rn(d2, d);
+    f[0] = __fadd2_rn(f[0], d);
+    f[1] = __fadd2_rn(f[1], d2);
+    f[2] = __fadd2_rn(f[2], d3);
+    f[3] = __ffma2_rn(d2, d2, f[3]);
+    f[4] = __ffma2_rn(d2, d3, f[4]);
+    f[5] = __ffma2_rn(d3, d3, f[5]);
+  };
+  if (slice < slices && r <= rmax) {
+    if (along_x) {
+      // runs of 32 positions of four rows
+      for (int k = slice; k < (h + 31) / 32 * (SF_LINES / 4); k += slices) {
+        const int j0 = k / (SF_LINES / 4) * 32, n = min(32, h - j0);
+        const float *s0 = strip + j0 * SF_STRIDE + 4 * (k % (SF_LINES / 4));
+        const float *s1 = s0 + r * SF_STRIDE;
+        float2 f[2][6];
+#pragma unroll
+        for (int p = 0; p < 6; ++p) f[0][p] = f[1][p] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) {
+          const float4 a = *reinterpret_cast<const float4 *>(s1 + j * SF_STRIDE);
+          const float4 b = *reinterpret_cast<const float4 *>(s0 + j * SF_STRIDE);
+          add(f[0], __ffma2_rn(make_float2(b.x, b.y), m1, make_float2(a.x, a.y)));
+          add(f[1], __ffma2_rn(make_float2(b.z, b.w), m1, make_float2(a.z, a.w)));
+        }
+#pragma unroll
+        for (int p = 0; p < 6; ++p) {
+          pair_add(hi[p], lo[p], f[0][p]);
+          pair_add(hi[p], lo[p], f[1][p]);
+        }
+      }
+    } else {
+      // 32 columns of two positions
+      for (int j = 2 * slice; j < h; j += 2 * slices) {
+        const float *s0 = strip + j, *s1 = s0 + r;
+        const bool two = j + 1 < h;
+        float2 f[6];
+#pragma unroll
+        for (int p = 0; p < 6; ++p) f[p] = make_float2(0.f, 0.f);
+#pragma unroll 8
+        for (int c = 0; c < SF_LINES; ++c) {
+          float2 d = __ffma2_rn(make_float2(s0[c * ystride], s0[c * ystride + 1]), m1,
+                                make_float2(s1[c * ystride], s1[c * ystride + 1]));
+          if (!two) d.y = 0.f;
+          add(f, d);
+        }
+#pragma unroll
+        for (int p = 0; p < 6; ++p) pair_add(hi[p], lo[p], f[p]);
       }
     }
   }
-  if (r <= rmax) {
-    double *o = part + ((size_t)(blockIdx.y * gridDim.x + blockIdx.x) * rmax + (r - 1)) * 6;
+  double acc[6];
+  bool finite = true;
 #pragma unroll
-    for (int p = 0; p < 6; ++p) o[p] = a.acc[p];
+  for (int p = 0; p < 6; ++p) {
+    acc[p] = ((double)hi[p].x + (double)hi[p].y) + ((double)lo[p].x + (double)lo[p].y);
+    finite &= isfinite(acc[p]);
   }
-}
-
-__global__ void __launch_bounds__(SFT_R)
-    k_sf_cols(const float *__restrict__ uy, int nx, int ny, int rmax, size_t part_off,
-              double *__restrict__ part) {
-  extern __shared__ float strip[];  // (SFT_Y + rmax) rows x SFT_CS
-  const int x0 = blockIdx.x * SFT_C, cw = min(SFT_C, nx - x0);
-  const int y0 = blockIdx.y * SFT_Y, h = min(SFT_Y, ny - y0);
-  const float *u = uy + (size_t)blockIdx.z * nx * ny;
-  for (int e = threadIdx.x; e < (h + rmax) * SFT_C; e += SFT_R) {
-    const int j = e / SFT_C, c = e % SFT_C;
-    if (c < cw) strip[j * SFT_CS + c] = u[(size_t)((y0 + j) % ny) * nx + x0 + c];
-  }
-  __syncthreads();
-  const int r = threadIdx.x + 1;
-  SfAcc a;
-  a.zero();
-  if (r <= rmax) {
+  if (!finite && slice < slices && r <= rmax) {
+    // a blown-up field: the FP32 running sums may overflow where FP64 ones do
+    // not, and two-sum turns an infinity into a NaN; add up in FP64 instead
+#pragma unroll
+    for (int p = 0; p < 6; ++p) acc[p] = 0.0;
+    const int sp = along_x ? SF_STRIDE : 1, sl = along_x ? 1 : ystride;
     for (int j = 0; j < h; ++j) {
-      const float *s0 = strip + j * SFT_CS, *s1 = strip + (j + r) * SFT_CS;
-      for (int c = 0; c < cw; ++c) a.add(s1[c] - s0[c]);
-      a.flush();
+      for (int l = 0; l < SF_LINES; ++l) {
+        // the nodes this slice took above
+        if ((along_x ? j / 32 * (SF_LINES / 4) + l / 4 : j / 2) % slices != slice) continue;
+        const float d = strip[(j + r) * sp + l * sl] - strip[j * sp + l * sl];
+        float q = d;
+        for (int p = 0; p < 6; ++p, q *= d) acc[p] += (double)q;
+      }
     }
-    const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    double *o = part + ((part_off + blk) * rmax + (r - 1)) * 6;
+  }
+  // slices in order, then one row of 6 x rmax partial sums per block
+  if (slices > 1) {
+    __syncthreads();  // the strip is read; its space takes the slices' sums
+    double *red = reinterpret_cast<double *>(strip);  // [slices][6][rt]
+    if (slice < slices)
 #pragma unroll
-    for (int p = 0; p < 6; ++p) o[p] = a.acc[p];
+      for (int p = 0; p < 6; ++p) red[(slice * 6 + p) * rt + r - 1] = acc[p];
+    __syncthreads();
+    if (slice == 0)
+      for (int k = 1; k < slices; ++k)
+#pragma unroll
+        for (int p = 0; p < 6; ++p) acc[p] += red[(k * 6 + p) * rt + r - 1];
+  }
+  if (slice == 0 && r <= rmax)
+#pragma unroll
+    for (int p = 0; p < 6; ++p) part[((size_t)blockIdx.x * 6 + p) * rmax + r - 1] = acc[p];
+}
+
+// out[e] = scale * sum over k (in a fixed order) of rows[k][e]: 32 columns per
+// block, the rows in 32 interleaved slices.
+constexpr int SUM_SLICES = 32;
+__global__ void __launch_bounds__(32 * SUM_SLICES)
+    k_sum_rows(const double *__restrict__ rows, int n, int width, double scale,
+               double *__restrict__ out) {
+  __shared__ double red[SUM_SLICES][33];
+  const int lane = threadIdx.x % 32, slice = threadIdx.x / 32;
+  const int e = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (e < width)
+#pragma unroll 4
+    for (int k = slice; k < n; k += SUM_SLICES) s += rows[(size_t)k * width + e];
+  red[slice][lane] = s;
+  __syncthreads();
+  if (slice == 0 && e < width) {
+    for (int k = 1; k < SUM_SLICES; ++k) s += red[k][lane];
+    out[e] = s * scale;
   }
 }
 
-// S[p][r] = sum over the blocks of the tiled form (in order) / (2 B N)
-__global__ void k_sf_final(const double *__restrict__ part, int rmax, int blocks,
-                           double inv_count, double *__restrict__ S) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= 6 * rmax) return;
-  const int p = e / rmax, r = e % rmax;
-  double s = 0.0;
-  for (int k = 0; k < blocks; ++k) s += part[((size_t)k * rmax + r) * 6 + p];
-  S[e] = s * inv_count;
-}
-
-struct SfTiles {
-  int xb, yb;  // blocks along x and y of the row kernel; of the column kernel: bx, by, bz
-  int cx, cy, cz;
-  __host__ int total() const { return xb * yb + cx * cy * cz; }
-};
-SfTiles sf_tiles(const Grid &g) {
-  SfTiles t;
-  t.xb = (g.nx + SFT_X - 1) / SFT_X;
-  t.yb = (g.ny * g.batch + SFT_RB - 1) / SFT_RB;
-  t.cx = (g.nx + SFT_C - 1) / SFT_C;
-  t.cy = (g.ny + SFT_Y - 1) / SFT_Y;
-  t.cz = g.batch;
-  return t;
+SfShape sf_shape(const Grid &g) {
+  SfShape s;
+  const long long rows = ((long long)g.ny * g.batch + SF_LINES - 1) / SF_LINES;
+  const long long strips = (long long)((g.nx + SF_LINES - 1) / SF_LINES) * g.batch;
+  // 32 positions per block (1,024 blocks per direction at 1024^2), up to 256
+  // while that leaves more than SF_MOST_BLOCKS rows of partial sums
+  for (s.h = 32;; s.h *= 2) {
+    s.segs_x = (g.nx + s.h - 1) / s.h;
+    s.segs_y = (g.ny + s.h - 1) / s.h;
+    const long long bx = rows * s.segs_x, by = strips * s.segs_y;
+    if (s.h == 256 || bx + by <= SF_MOST_BLOCKS) {
+      s.bx = bx + by <= 0x7fffffffLL ? (int)bx : 0;
+      s.by = bx + by <= 0x7fffffffLL ? (int)by : 0;
+      return s;
+    }
+  }
 }
 
 // S[p][r] = sum over chunks (in order) / (2 B N)
@@ -221,6 +293,13 @@ __global__ void k_structure_final(const double *__restrict__ part, int rmax, int
 
 __device__ __forceinline__ long long isqrt_floor(long long v) {
   if (v <= 0) return 0;
+  if (v < 1 << 24) {  // in single precision (FP64 roots took half of k_spectrum_rows)
+    const int w = (int)v;
+    int s = (int)sqrtf((float)w);
+    while (s * s > w) --s;
+    while ((s + 1) * (s + 1) <= w) ++s;
+    return s;
+  }
   long long s = (long long)sqrt((double)v);
   while (s * s > v) --s;
   while ((s + 1) * (s + 1) <= v) ++s;
@@ -255,25 +334,22 @@ __global__ void k_spectrum_rows(const cufftComplex *__restrict__ uh, int nx, int
   rowpart[(size_t)j * (kmax + 1) + s] = acc;
 }
 
-__global__ void k_spectrum_final(const double *__restrict__ rowpart, int ny, int kmax,
-                                 double scale, double *__restrict__ E) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s > kmax) return;
-  double acc = 0.0;
-  for (int j = 0; j < ny; ++j) acc += rowpart[(size_t)j * (kmax + 1) + s];
-  E[s] = acc * scale;
-}
-
 }  // namespace
 
-// The tiled form applies for rmax <= SFT_R and grids within its launch limits.
-static bool sf_tiled(const Grid &g, int rmax) {
-  const SfTiles t = sf_tiles(g);
-  return rmax <= SFT_R && t.yb <= 65535 && t.cy <= 65535 && t.cz <= 65535;
+// Positions of x or y increments, or the slices' sums (6 doubles per thread).
+static size_t sf_smem(int h, int rmax) {
+  const size_t n = sizeof(float) * (size_t)(h + rmax + 3) * SF_STRIDE;
+  return n > sizeof(double) * 6 * SFT_R ? n : sizeof(double) * 6 * SFT_R;
 }
 
+// The tiled form applies for rmax <= SFT_R and grids within its launch limits.
+static bool sf_tiled(const Grid &g, int rmax) { return rmax <= SFT_R && sf_shape(g).bx > 0; }
+
 size_t structure_partials_doubles(const Grid &g, int rmax) {
-  if (sf_tiled(g, rmax)) return (size_t)sf_tiles(g).total() * rmax * 6;
+  if (sf_tiled(g, rmax)) {
+    const SfShape s = sf_shape(g);
+    return (size_t)(s.bx + s.by) * rmax * 6;
+  }
   const int rows = g.ny * g.batch;
   const int rpb = 8;
   const int chunks = (rows + rpb - 1) / rpb;
@@ -283,25 +359,20 @@ size_t structure_partials_doubles(const Grid &g, int rmax) {
 cudaError_t launch_structure_functions(const Grid &g, const float *ux, const float *uy, int rmax,
                                        double *part, double *S, cudaStream_t s) {
   if (sf_tiled(g, rmax)) {
-    const SfTiles t = sf_tiles(g);
-    const size_t smem_cols = sizeof(float) * (size_t)(SFT_Y + rmax) * SFT_CS;
+    const SfShape sh = sf_shape(g);
     static bool attr_set = false;
     if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(k_sf_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(sizeof(float) * (SFT_Y + SFT_R) * SFT_CS));
+      cudaError_t e = cudaFuncSetAttribute(k_sf_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sf_smem(256, SFT_R));
       if (e != cudaSuccess) return e;
       attr_set = true;
     }
-    k_sf_rows<<<dim3(t.xb, t.yb), SFT_R, sizeof(float) * (SFT_X + rmax), s>>>(
-        ux, g.nx, g.ny * g.batch, rmax, part);
+    k_sf_strips<<<sh.bx + sh.by, SFT_R, sf_smem(sh.h, rmax), s>>>(ux, uy, g.nx, g.ny, g.batch,
+                                                                     rmax, sh, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_sf_cols<<<dim3(t.cx, t.cy, t.cz), SFT_R, smem_cols, s>>>(uy, g.nx, g.ny, rmax,
-                                                              (size_t)t.xb * t.yb, part);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_sf_final<<<(6 * rmax + 255) / 256, 256, 0, s>>>(part, rmax, t.total(),
-                                                      1.0 / (2.0 * (double)g.nodes()), S);
+    k_sum_rows<<<(6 * rmax + 31) / 32, 32 * SUM_SLICES, 0, s>>>(
+        part, sh.bx + sh.by, 6 * rmax, 1.0 / (2.0 * (double)g.nodes()), S);
     return cudaGetLastError();
   }
   const int rows = g.ny * g.batch;
@@ -340,8 +411,8 @@ cudaError_t launch_energy_spectrum(const Grid &g, float *u, void *uh, void **pla
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const double N = (double)g.nx * g.ny;
-  k_spectrum_final<<<(kmax + 1 + 127) / 128, 128, 0, s>>>(rowpart, g.ny, kmax,
-                                                          0.5 / (N * N * g.batch), E);
+  k_sum_rows<<<(kmax + 32) / 32, 32 * SUM_SLICES, 0, s>>>(rowpart, g.ny, kmax + 1,
+                                                         0.5 / (N * N * g.batch), E);
   return cudaGetLastError();
 }
 

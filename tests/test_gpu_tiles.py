@@ -103,3 +103,52 @@ def test_several_steps_per_launch(lbm, kind, nx, ny, B, n):  # noqa: F811
         assert (one.state_buffer() == one.bufs[0].data_ptr()) == \
             (many.state_buffer() == many.bufs[0].data_ptr())
         assert one.status() == many.status() == (lbm.LBM_ERR_UNSTABLE if fast else lbm.LBM_OK)
+
+
+@pytest.mark.parametrize("nx,ny,B,rmax", [(31, 33, 1, 40), (32, 64, 2, 64), (65, 31, 3, 7),
+                                          (300, 260, 1, 256), (1, 9, 1, 3)])
+def test_structure_function_strips(lbm, nx, ny, B, rmax):  # noqa: F811
+    """Structure functions on strips of 32 lines and several positions per block,
+    with ragged ends, more separations than the lattice is wide, and one or more
+    slices of threads: against FP64 sums over the same FP32 velocities.  Each
+    block's FP32 sums have at most 32 terms, so an entry is within 32 half-ulps
+    (2^-24) of its sum of absolute terms plus the three or fewer roundings per
+    term of its powers: 40 * 2^-24 of that sum."""
+    lat = lbm.Lattice(nx, ny, B, device=DEV)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(nx)
+    lat.set_state(torch.rand((B, 9, ny, nx), generator=g, device=DEV) * 0.01 + 0.1)
+    S = lat.structure_functions(rmax).cpu().numpy()
+    _, ux, uy = (t.cpu().numpy() for t in lat.moments())
+    for r in range(1, rmax + 1):
+        dx = (np.roll(ux, -r, axis=2) - ux).astype(float)
+        dy = (np.roll(uy, -r, axis=1) - uy).astype(float)
+        for p in range(1, 7):
+            ref = 0.5 * np.mean(dx ** p + dy ** p)
+            tol = 40 * 2.0 ** -24 * 0.5 * np.mean(np.abs(dx) ** p + np.abs(dy) ** p)
+            assert abs(S[p - 1, r - 1] - ref) <= tol, (p, r)
+
+
+def test_structure_functions_of_a_blown_up_field(lbm):  # noqa: F811
+    """Velocities so large that FP32 running sums overflow: the sums of the even
+    powers stay the finite FP64 ones; with an infinite velocity no sum is finite."""
+    nx, ny, rmax = 64, 96, 40
+    g = torch.Generator(device=DEV)
+    g.manual_seed(3)
+    ux, uy = ((torch.rand((1, ny, nx), generator=g, device=DEV) - 0.5) * 2e6 for _ in range(2))
+    f = torch.zeros((1, 9, ny, nx), device=DEV)
+    f[:, 0] = 1.0
+    f[:, 1], f[:, 3] = ux / 2, -ux / 2   # rho = 1, j = (ux, uy)
+    f[:, 2], f[:, 4] = uy / 2, -uy / 2
+    lat = lbm.Lattice(nx, ny, 1, device=DEV)
+    lat.set_state(f)
+    _, vx, vy = (t.cpu().numpy().astype(float) for t in lat.moments())
+    S = lat.structure_functions(rmax).cpu().numpy()
+    for r in (1, 7, rmax):
+        dx, dy = np.roll(vx, -r, axis=2) - vx, np.roll(vy, -r, axis=1) - vy
+        for p in (2, 4, 6):
+            ref = 0.5 * np.mean(dx ** p + dy ** p)
+            assert abs(S[p - 1, r - 1] / ref - 1) <= 40 * 2.0 ** -24
+    f[0, 1, 5, 6] = float("inf")
+    lat.set_state(f)
+    assert not np.isfinite(lat.structure_functions(rmax).cpu().numpy()).any()
