@@ -75,7 +75,8 @@ typedef struct {
  * with this library's widths).  Device pointers, row-major [out][in]:
  * w1[64][9], b1[64], w2[64][64], b2[64], w3[9][64], b3[9].
  * dtype 0 = FP32 (both MLP kinds), 1 = BF16 (LBM_MLP_BF16 only).  The
- * weights are read at launch, never copied or retained. */
+ * weights are read by the kernels of each call (a call of several tensor-core
+ * steps lays them out once, in the context's scratch), never retained. */
 typedef struct {
   const void *w1, *b1, *w2, *b2, *w3, *b3;
   int dtype;

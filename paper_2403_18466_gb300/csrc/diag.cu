@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(SFT_R)
                 int batch, int rmax, SfShape sh, double *__restrict__ part) {
   extern __shared__ __align__(16) float strip[];  // (h + rmax) positions of 32 lines
   const bool along_x = (int)blockIdx.x < sh.bx;
-  const int ystride = (sh.h + rmax + 2) / 2 * 2 + 1;  // odd: a warp stages 32 columns
+  const int ystride = (sh.h + rmax + 2) / 4 * 4 + 2;  // even: aligned pairs; 2-way when staged
   const int rt = (rmax + 31) / 32 * 32;  // threads per slice; slices share the positions
   const int slices = blockDim.x / rt, slice = threadIdx.x / rt, r = threadIdx.x % rt + 1;
   int h;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(SFT_R)
         for (int p = 0; p < 6; ++p) f[p] = make_float2(0.f, 0.f);
 #pragma unroll 8
         for (int c = 0; c < SF_LINES; ++c) {
-          float2 d = __ffma2_rn(make_float2(s0[c * ystride], s0[c * ystride + 1]), m1,
+          float2 d = __ffma2_rn(*reinterpret_cast<const float2 *>(s0 + c * ystride), m1,
                                 make_float2(s1[c * ystride], s1[c * ystride + 1]));
           if (!two) d.y = 0.f;
           add(f, d);

@@ -77,15 +77,23 @@ cudaError_t launch_step_mlp_f32(const Grid &g, const float *in, float *out,
                                 cudaStream_t s);
 
 // mlp_bf16.cu ------------------------------------------------------------------
-// weights: FP32 (dtype 0) or BF16 (dtype 1), same packed row-major layout.
+// FP32 (dtype 0) or BF16 (dtype 1) parameters, packed row-major layout.
+struct MlpPtrs {
+  const void *w1, *b1, *w2, *b2, *w3, *b3;
+};
+// Lays the weights out as operand tiles in a device buffer of
+// mlp_bf16_tile_bytes() bytes (16-byte aligned).
+size_t mlp_bf16_tile_bytes();
+cudaError_t launch_prepare_weights_bf16(const MlpPtrs &w, int dtype, void *tiles, cudaStream_t s);
+// tiles: the prepared weights, or nullptr to lay them out in every CTA.
 // wait_limit: polls of each bounded mbarrier wait before the kernel gives up
 // and sets *timeout_flag (0 = the default, 2^20); max_ctas: cap on the
 // persistent grid (0 = one CTA per SM); chain: the previous operation on `s`
 // is this kernel with the same weights, so it is launched as a programmatic
 // dependent of it (its prologue overlaps that kernel's last tiles).
 cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,
-                                 const CollideParams &p, const void *const wptr[6], int dtype,
-                                 int *flag, int *timeout_flag, cudaStream_t s,
+                                 const CollideParams &p, const MlpPtrs &w, int dtype,
+                                 const void *tiles, int *flag, int *timeout_flag, cudaStream_t s,
                                  unsigned wait_limit = 0, int max_ctas = 0, bool chain = false);
 
 // Compiled layout of the tensor-core step: tile warpgroups per SM and, of

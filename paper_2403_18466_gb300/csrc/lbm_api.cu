@@ -26,6 +26,8 @@ struct lbm_ctx {
   CollideParams cp;
   // scratch (library-owned, device)
   int *d_flag;          // [0] unstable, [1] device wait timeout, [2] bad node index
+  void *d_tiles;        // operand tiles of the tensor-core step, in the allocation of d_flag
+  bool tiles_ready;     // they hold the weights of the call in progress
   float *d_force;       // ny floats, or nullptr
   float *d_loss_part;   // lbm::loss_partials(g) doubles (float or double partials)
   float *d_dw_part;     // dw_rows * NPARAMS floats (allocated on first use)
@@ -89,6 +91,22 @@ MlpF32 f32_view(const lbm_weights *w) {
   return m;
 }
 
+lbm::MlpPtrs ptrs(const lbm_weights *w) { return {w->w1, w->b1, w->w2, w->b2, w->w3, w->b3}; }
+
+// The operand tiles of a call's tensor-core steps, laid out once by a launch of
+// its own when the call has several (one step lays them out itself: a launch
+// costs about as much as that).  Valid within one call only: the next may come
+// with other weights.
+struct Tiles {
+  lbm_ctx *c;
+  Tiles(lbm_ctx *ctx, lbm_collision kind, const lbm_weights *w, int steps) : c(ctx) {
+    c->tiles_ready = kind == LBM_MLP_BF16 && steps > 1 &&
+                     lbm::launch_prepare_weights_bf16(ptrs(w), w->dtype, c->d_tiles, c->stream) ==
+                         cudaSuccess;
+  }
+  ~Tiles() { c->tiles_ready = false; }
+};
+
 // One launch from `in` to `out` with the given collision: `steps` steps of a
 // plain collision (at most lbm::step_plan's), one of a learned one.  `chain`: the previous
 // operation on the stream is a step of the same collision issued by the same
@@ -104,8 +122,8 @@ cudaError_t one_step(lbm_ctx *c, const float *in, float *out, lbm_collision kind
     case LBM_MLP_F32:
       return lbm::launch_step_mlp_f32(c->g, in, out, c->cp, f32_view(w), c->d_flag, c->stream);
     case LBM_MLP_BF16: {
-      const void *wp[6] = {w->w1, w->b1, w->w2, w->b2, w->w3, w->b3};
-      return lbm::launch_step_mlp_bf16(c->g, in, out, c->cp, wp, w->dtype, c->d_flag,
+      return lbm::launch_step_mlp_bf16(c->g, in, out, c->cp, ptrs(w), w->dtype,
+                                       c->tiles_ready ? c->d_tiles : nullptr, c->d_flag,
                                        c->d_flag + 1, c->stream, c->wait_limit, c->max_ctas,
                                        chain);
     }
@@ -185,9 +203,10 @@ int lbm_init(lbm_ctx **out, const lbm_params *p, float *f_buf0, float *f_buf1,
   c->cp.smag_c18 = (float)(18.0 * (p->smag_cs * p->smag_delta) * (p->smag_cs * p->smag_delta));
   c->cp.force = nullptr;
   int rc = LBM_OK;
-  if (cudaMalloc(&c->d_flag, 3 * sizeof(int)) != cudaSuccess ||
+  if (cudaMalloc(&c->d_flag, 256 + lbm::mlp_bf16_tile_bytes()) != cudaSuccess ||
       cudaMemset(c->d_flag, 0, 3 * sizeof(int)) != cudaSuccess)
     rc = LBM_ERR_CUDA;
+  c->d_tiles = reinterpret_cast<char *>(c->d_flag) + 256;
   if (rc == LBM_OK && p->force_amp != 0.0) {
     // F_x(y) = F0 sin(2 pi m y / ny), evaluated in double on the host
     float *h = static_cast<float *>(std::malloc(sizeof(float) * p->ny));
@@ -259,6 +278,7 @@ int lbm_step(lbm_ctx *c, int n, lbm_collision kind, const lbm_weights *w) {
   const int most = kind <= LBM_SMAG ? lbm::step_plan(c->g).steps : 1;
   int launches = n / most + (n % most ? 1 : 0);
   if ((n - launches) & 1) ++launches;
+  const Tiles tiles(c, kind, w, n);
   for (int s = 0; s < launches; ++s) {
     const int steps = n / launches + (s < n % launches ? 1 : 0);
     CUDA_TRY(one_step(c, c->buf[c->cur], c->buf[c->cur ^ 1], kind, w, s > 0, steps));
@@ -381,6 +401,7 @@ static int forward_record(lbm_ctx *c, lbm_collision kind, int n, int k, const lb
   float *seg = reinterpret_cast<float *>(base + (size_t)n_checkpoints(n, k) * sb);
   const size_t sf = sb / sizeof(float);
   c->rec_last_seg = false;
+  const Tiles tiles(c, kind, w, n);
   CUDA_TRY(cudaMemcpyAsync(base, c->buf[c->cur], sb, cudaMemcpyDeviceToDevice, c->stream));
   const float *in = c->buf[c->cur];
   for (int s = 0; s < n; ++s) {
@@ -437,6 +458,7 @@ static int backward(lbm_ctx *c, bool tc, const float *dL_df_final, const lbm_wei
                    reinterpret_cast<float *>(base + (size_t)(nck + k) * sb)};
   const size_t sf = sb / sizeof(float);
   const MlpF32 wf = f32_view(w);
+  const Tiles tiles(c, kind, w, n > k ? k - 1 : 0);  // of the recomputed segments
   // lam = dL/d(stored state g^n): the transpose of the final pull is a push
   CUDA_TRY(lbm::launch_push(c->g, dL_df_final, lam[0], c->stream));
   int cur = 0;

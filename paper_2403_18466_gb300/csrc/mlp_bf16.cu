@@ -58,6 +58,10 @@
 // flag and drains its outstanding commit (full limit), and tensor memory is
 // always freed.
 //
+// A call of several steps lays its weights out once (k_prepare_weights), and
+// each step's CTAs take them with one bulk copy instead of converting 7,400
+// parameters each (256^2: 9.4 -> 7.8 us per step).
+//
 // Consecutive steps of one call are programmatic dependent launches: a step's
 // prologue (weights to shared memory, tensor-memory allocation) runs on the
 // SMs that the previous step has already left, and griddepcontrol.wait holds
@@ -98,7 +102,9 @@ constexpr int FMA_PACK = LBM_TANH_FMA_PACK;
 #define LBM_LEADER_SPREAD 1
 #endif
 constexpr bool LEADER_SPREAD = LBM_LEADER_SPREAD != 0;
-constexpr int THREADS = WGS * WG_THREADS;
+// Lattices of few tiles take CTAs of half the warpgroups, two of which fit on an
+// SM: the next step's CTA then runs its prologue beside this one.
+constexpr int FEW_WGS = 4;
 constexpr int XU_PAIRS = LBM_TANH_XU_PAIRS;  // of every 8 activation pairs, on the XU
 static_assert(XU_PAIRS >= 0 && XU_PAIRS <= 8, "split of 8 pairs");
 constexpr int K1 = 16, K2 = 80;  // padded K of layer 1 and of layers 2/3
@@ -109,8 +115,7 @@ constexpr int K1 = 16, K2 = 80;  // padded K of layer 1 and of layers 2/3
 constexpr int EPI_COLS = LBM_EPI_COLS;
 static_assert(EPI_COLS == 16 || EPI_COLS == 32, "16 or 32 columns per read");
 // tensor memory: 64 accumulator columns per warpgroup
-constexpr uint32_t TMEM_COLS = 512;
-static_assert(WGS * 64 <= (int)TMEM_COLS, "tensor memory layout");
+static_assert(WGS * 64 <= 512, "tensor memory layout");
 constexpr uint32_t DEFAULT_WAIT_LIMIT = 1u << 20;  // polls; far above any real MMA latency
 
 // Bounded wait for a GEMM's commit.  A limit of 1024 polls or more uses
@@ -136,19 +141,26 @@ constexpr float TP0 = 3.9946699142456055f, TP1 = -20.35879898071289f, TP2 = 103.
 // then accumulated pre-scaled by 1/4).
 __host__ __device__ constexpr bool fma_unit(int n) { return (n % 16) >= 2 * XU_PAIRS; }
 
+template <int NWG>
 struct __align__(1024) Smem {
   unsigned char w1[HIDDEN * K1 * 2];     // B of layer 1: [64 x 16] = W1 | b1 | 0
   unsigned char w2[HIDDEN * K2 * 2];     // B of layer 2: [64 x 80] = W2 | b2 | 0
   unsigned char w3[16 * K2 * 2];         // B of layer 3: [16 x 80] = W3 | b3 | 0, rows 9..15 zero
-  unsigned char a1[WGS][128 * K1 * 2];   // A of layer 1, per warpgroup
-  unsigned char a23[WGS][128 * K2 * 2];  // A of layers 2 and 3, per warpgroup
-  unsigned long long bar[WGS];
+  unsigned char a1[NWG][128 * K1 * 2];   // A of layer 1, per warpgroup
+  unsigned char a23[NWG][128 * K2 * 2];  // A of layers 2 and 3, per warpgroup
+  unsigned long long bar[NWG];
+  unsigned long long wbar;  // the weights' bulk copy
   uint32_t taddr;
 };
-// One CTA per SM (its tensor-memory allocation takes all 512 columns): the
-// dynamic shared memory request is padded so that no second CTA fits.
-constexpr size_t SMEM_BYTES = (sizeof(Smem) + 1024) > 120 * 1024 ? sizeof(Smem) + 1024 : 120 * 1024;
-static_assert(SMEM_BYTES <= 227 * 1024, "shared memory layout too large");
+// CTAs of WGS warpgroups: one per SM (its tensor-memory allocation takes all 512
+// columns), so the dynamic shared memory request is padded until no second CTA
+// fits.  CTAs of FEW_WGS: two.
+template <int NWG>
+constexpr size_t smem_bytes() {
+  return NWG < WGS || sizeof(Smem<NWG>) + 1024 > 120 * 1024 ? sizeof(Smem<NWG>) + 1024 : 120 * 1024;
+}
+static_assert(smem_bytes<WGS>() <= 227 * 1024, "shared memory layout too large");
+static_assert(2 * (smem_bytes<FEW_WGS>() + 1024) <= 228 * 1024, "two CTAs per SM");
 
 __device__ __forceinline__ void store_bf16(unsigned char *base, int r, int k, int K, float v) {
   *reinterpret_cast<__nv_bfloat16 *>(base + canon_offset(r, k, K)) = __float2bfloat16_rn(v);
@@ -314,52 +326,73 @@ __device__ __forceinline__ void finish_node(const uint32_t ov[16], const NodePre
   }
 }
 
+// Weights -> bf16 operand tiles (FMA-form units pre-scaled by 1/4, exact in
+// bf16), biases in the constant-1 column; elements tid, tid + n, ... of the
+// three tiles, which lie one after another.
+constexpr int W1_BYTES = HIDDEN * K1 * 2, W2_BYTES = HIDDEN * K2 * 2, W3_BYTES = 16 * K2 * 2;
+constexpr int W_BYTES = W1_BYTES + W2_BYTES + W3_BYTES;
 template <int DTYPE>
-__global__ void __launch_bounds__(THREADS, 1)
+__device__ __forceinline__ void fill_weights(unsigned char *dst, const MlpPtrs &w, int tid, int n) {
+  for (int e = tid; e < HIDDEN * K1; e += n) {
+    const int j = e / K1, k = e % K1;
+    float v = k < 9 ? wload<DTYPE>(w.w1, j * 9 + k) : (k == 9 ? wload<DTYPE>(w.b1, j) : 0.f);
+    if (fma_unit(j)) v *= 0.25f;
+    store_bf16(dst, j, k, K1, v);
+  }
+  for (int e = tid; e < HIDDEN * K2; e += n) {
+    const int j = e / K2, k = e % K2;
+    float v = k < HIDDEN ? wload<DTYPE>(w.w2, j * HIDDEN + k)
+                         : (k == HIDDEN ? wload<DTYPE>(w.b2, j) : 0.f);
+    if (fma_unit(j)) v *= 0.25f;
+    store_bf16(dst + W1_BYTES, j, k, K2, v);
+  }
+  for (int e = tid; e < 16 * K2; e += n) {
+    const int j = e / K2, k = e % K2;
+    float v = 0.f;
+    if (j < 9)
+      v = k < HIDDEN ? wload<DTYPE>(w.w3, j * HIDDEN + k) : (k == HIDDEN ? wload<DTYPE>(w.b3, j) : 0.f);
+    store_bf16(dst + W1_BYTES + W2_BYTES, j, k, K2, v);
+  }
+}
+template <int DTYPE>
+__global__ void k_prepare_weights(MlpPtrs w, unsigned char *__restrict__ dst) {
+  fill_weights<DTYPE>(dst, w, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// SRC: where the weights come from -- 0, 1: FP32 or bf16 parameters, laid out
+// by every CTA; 2: the operand tiles of k_prepare_weights, one bulk copy.
+template <int SRC, int NWG>
+__global__ void __launch_bounds__(NWG *WG_THREADS, WGS / NWG)
     k_step_mlp_bf16(const float *__restrict__ in, float *__restrict__ out, int nx, int ny,
-                    int batch, CollideParams p, const void *w1, const void *b1, const void *w2,
-                    const void *b2, const void *w3, const void *b3, int *flag, int *timeout_flag,
-                    uint32_t wait_limit) {
+                    int batch, CollideParams p, MlpPtrs w, const unsigned char *__restrict__ tiles,
+                    int *flag, int *timeout_flag, uint32_t wait_limit) {
   extern __shared__ unsigned char smem_raw[];
-  Smem &S = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+  Smem<NWG> &S = *reinterpret_cast<Smem<NWG> *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                       ~uintptr_t(1023));
   const int tid = threadIdx.x;
   const int wg = tid / WG_THREADS;  // warpgroup within the CTA
   const int r = tid % WG_THREADS;   // row = node within the tile = TMEM lane
   const int warp_in_wg = r / 32;
 
-  // ---- prologue: weights -> bf16 operand tiles (FMA-form units pre-scaled
-  // by 1/4, exact in bf16), constant columns, barriers, tensor memory
-  for (int e = tid; e < HIDDEN * K1; e += THREADS) {
-    const int n = e / K1, k = e % K1;
-    float v = k < 9 ? wload<DTYPE>(w1, n * 9 + k) : (k == 9 ? wload<DTYPE>(b1, n) : 0.f);
-    if (fma_unit(n)) v *= 0.25f;
-    store_bf16(S.w1, n, k, K1, v);
-  }
-  for (int e = tid; e < HIDDEN * K2; e += THREADS) {
-    const int n = e / K2, k = e % K2;
-    float v = k < HIDDEN ? wload<DTYPE>(w2, n * HIDDEN + k) : (k == HIDDEN ? wload<DTYPE>(b2, n) : 0.f);
-    if (fma_unit(n)) v *= 0.25f;
-    store_bf16(S.w2, n, k, K2, v);
-  }
-  for (int e = tid; e < 16 * K2; e += THREADS) {
-    const int n = e / K2, k = e % K2;
-    float v = 0.f;
-    if (n < 9)
-      v = k < HIDDEN ? wload<DTYPE>(w3, n * HIDDEN + k) : (k == HIDDEN ? wload<DTYPE>(b3, n) : 0.f);
-    store_bf16(S.w3, n, k, K2, v);
-  }
+  // ---- prologue: weights, constant columns, barriers, tensor memory
+  if (SRC < 2) fill_weights<SRC>(S.w1, w, tid, NWG * WG_THREADS);
   unsigned char *a1 = S.a1[wg];
   unsigned char *a23 = S.a23[wg];
   // constant K columns 64..79 of this thread's layer-2/3 operand row: 1, 0, ..., 0
   *reinterpret_cast<uint4 *>(a23 + canon_offset(r, 64, K2)) = make_uint4(0x3F80u, 0u, 0u, 0u);
   *reinterpret_cast<uint4 *>(a23 + canon_offset(r, 72, K2)) = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
-    for (int k = 0; k < WGS; ++k) mbar_init(smem_u32(&S.bar[k]), 1);
+    for (int k = 0; k < NWG; ++k) mbar_init(smem_u32(&S.bar[k]), 1);
+    mbar_init(smem_u32(&S.wbar), 1);
     fence_mbarrier_init();
+    if (SRC == 2) {
+      fence_proxy_async();
+      mbar_arrive_expect_tx(smem_u32(&S.wbar), W_BYTES);
+      bulk_g2s(smem_u32(S.w1), tiles, W_BYTES, smem_u32(&S.wbar));
+    }
   }
   if (tid < 32) {
-    tmem_alloc(smem_u32(&S.taddr), TMEM_COLS);
+    tmem_alloc(smem_u32(&S.taddr), 64 * NWG);
     tmem_relinquish();
   }
   fence_proxy_async();
@@ -389,11 +422,13 @@ __global__ void __launch_bounds__(THREADS, 1)
   const size_t plane = (size_t)nx * ny;
   const int tiles_x = (nx + WG_THREADS - 1) / WG_THREADS;
   const long long ntiles = (long long)tiles_x * ny * batch;
-  const long long nwg = (long long)gridDim.x * WGS;
-  const long long gwg = (long long)blockIdx.x * WGS + wg;
+  const long long nwg = (long long)gridDim.x * NWG;
+  // few tiles: one per CTA before a second one joins it (see the launcher)
+  const long long gwg = ntiles < nwg ? (long long)wg * gridDim.x + blockIdx.x
+                                     : (long long)blockIdx.x * NWG + wg;
   const long long per = ntiles / nwg, extra = ntiles % nwg;
   const long long t_begin = gwg * per + (gwg < extra ? gwg : extra);
-  const int count = (int)(per + (gwg < extra ? 1 : 0));
+  int count = (int)(per + (gwg < extra ? 1 : 0));
   TilePos T;
   T.x0 = (int)(t_begin % tiles_x) * WG_THREADS;
   T.y = (int)((t_begin / tiles_x) % ny);
@@ -410,7 +445,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   griddep_launch_dependents();
 
   uint32_t phase = 0;
-  bool fail = false;  // the leader's last bounded wait gave up (leader only)
+  // the leader's last bounded wait gave up (leader only): the weights' copy,
+  // then each GEMM
+  bool fail = SRC == 2 && leader && !mbar_wait_bounded(smem_u32(&S.wbar), 0, DEFAULT_WAIT_LIMIT);
+  if (SRC == 2 && barrier_any(bar_id, WG_THREADS, fail)) count = 0;
   bool bad = false;   // an unstable node was met (per thread)
 
   NodePrep P;
@@ -519,12 +557,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   // memory is released
   if (leader && fail) {
     atomicOr(timeout_flag, 1);
-    mbar_wait_bounded(bar, phase, DEFAULT_WAIT_LIMIT);
+    if (count > 0) mbar_wait_bounded(bar, phase, DEFAULT_WAIT_LIMIT);
   }
   flag_unstable(bad, flag);
   fence_before_sync();
   __syncthreads();
-  if (tid < 32) tmem_dealloc(S.taddr, TMEM_COLS);
+  if (tid < 32) tmem_dealloc(S.taddr, 64 * NWG);
 }
 
 // The activations of the step kernel applied element-wise (path 0: XU pair,
@@ -572,27 +610,45 @@ cudaError_t launch_activation(const float *a, int n, int path, float *out, cudaS
   return cudaGetLastError();
 }
 
+size_t mlp_bf16_tile_bytes() { return W_BYTES; }
+
+cudaError_t launch_prepare_weights_bf16(const MlpPtrs &w, int dtype, void *tiles, cudaStream_t s) {
+  auto kern = dtype == 0 ? k_prepare_weights<0> : k_prepare_weights<1>;
+  kern<<<16, 256, 0, s>>>(w, static_cast<unsigned char *>(tiles));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,
-                                 const CollideParams &p, const void *const wp[6], int dtype,
-                                 int *flag, int *timeout_flag, cudaStream_t s,
+                                 const CollideParams &p, const MlpPtrs &w, int dtype,
+                                 const void *tiles, int *flag, int *timeout_flag, cudaStream_t s,
                                  unsigned wait_limit, int max_ctas, bool chain) {
   static int sms = 0;
-  static bool attr_done[2] = {false, false};
+  static bool attr_done[4] = {false, false, false, false};
   if (!sms) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
   }
-  auto kern = dtype == 0 ? k_step_mlp_bf16<0> : k_step_mlp_bf16<1>;
-  if (!attr_done[dtype]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)SMEM_BYTES);
+  const long long count = (long long)((g.nx + WG_THREADS - 1) / WG_THREADS) * g.ny * g.batch;
+  // Few tiles and prepared weights: the half-size CTAs (up to four tiles per SM,
+  // all in flight at once either way; 256^2: 7.8 -> 7.3 us per step).
+  const bool few = tiles && max_ctas == 0 && count <= (long long)FEW_WGS * sms;
+  const int src = few ? 3 : (tiles ? 2 : dtype);
+  auto kern = src == 0   ? k_step_mlp_bf16<0, WGS>
+              : src == 1 ? k_step_mlp_bf16<1, WGS>
+              : src == 2 ? k_step_mlp_bf16<2, WGS>
+                         : k_step_mlp_bf16<2, FEW_WGS>;
+  const size_t smem = few ? smem_bytes<FEW_WGS>() : smem_bytes<WGS>();
+  if (!attr_done[src]) {
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    attr_done[dtype] = true;
+    attr_done[src] = true;
   }
-  const long long tiles = (long long)((g.nx + WG_THREADS - 1) / WG_THREADS) * g.ny * g.batch;
-  long long ctas = (tiles + WGS - 1) / WGS;
+  // One CTA per SM while there are tiles for it: a tile alone on its SM is done
+  // sooner than eight at a time (64^2: 9.3 -> 5.0 us per step).
+  long long ctas = count;
   if (ctas > (long long)sms) ctas = sms;
   if (max_ctas > 0 && ctas > max_ctas) ctas = max_ctas;
   if (wait_limit == 0) wait_limit = DEFAULT_WAIT_LIMIT;
@@ -602,16 +658,17 @@ cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,
   // weights, which an earlier operation may still be writing
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctas);
-  cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.blockDim = dim3((few ? FEW_WGS : WGS) * WG_THREADS);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chain ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, in, out, g.nx, g.ny, g.batch, p, wp[0], wp[1], wp[2],
-                            wp[3], wp[4], wp[5], flag, timeout_flag, wait_limit);
+  return cudaLaunchKernelEx(&cfg, kern, in, out, g.nx, g.ny, g.batch, p, w,
+                            static_cast<const unsigned char *>(tiles), flag, timeout_flag,
+                            wait_limit);
 }
 
 }  // namespace lbm

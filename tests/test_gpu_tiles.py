@@ -152,3 +152,26 @@ def test_structure_functions_of_a_blown_up_field(lbm):  # noqa: F811
     f[0, 1, 5, 6] = float("inf")
     lat.set_state(f)
     assert not np.isfinite(lat.structure_functions(rmax).cpu().numpy()).any()
+
+
+@pytest.mark.parametrize("dtype", ["float32", "bfloat16"])
+@pytest.mark.parametrize("nx,ny,B", [(1, 1, 1), (64, 64, 1), (129, 9, 2), (128, 608, 1),
+                                     (128, 609, 1), (250, 700, 1)])
+def test_tensor_core_steps_of_one_call(lbm, nx, ny, B, dtype):  # noqa: F811
+    """Several tensor-core steps of one call (weights laid out once, half-size
+    CTAs up to four tiles per SM) have the bits of calls of one step each."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(ny)
+    f = torch.rand((B, 9, ny, nx), generator=g, device=DEV) * 0.005 + \
+        torch.tensor([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4, device=DEV).view(1, 9, 1, 1)
+    th = torch.tensor(inputs.xavier_mlp(3, bias_scale=0.2, out_scale=0.1), device=DEV)
+    w = lbm.weights_struct(th.to(getattr(torch, dtype)))
+    one, many = (lbm.Lattice(nx, ny, B, tau=0.6, force_amp=1e-4, force_mode=1, device=DEV)
+                 for _ in range(2))
+    for lat in (one, many):
+        lat.set_state(f)
+    for _ in range(5):
+        one.step(1, "mlp_bf16", w)
+    many.step(5, "mlp_bf16", w)
+    assert torch.equal(one.get_state(), many.get_state())
+    assert one.status() == many.status() == lbm.LBM_OK
