@@ -175,3 +175,35 @@ def test_tensor_core_steps_of_one_call(lbm, nx, ny, B, dtype):  # noqa: F811
     many.step(5, "mlp_bf16", w)
     assert torch.equal(one.get_state(), many.get_state())
     assert one.status() == many.status() == lbm.LBM_OK
+
+
+@pytest.mark.parametrize("nx,ny,B", [(1, 1, 1), (127, 1, 1), (43, 3, 1), (16, 8, 2), (257, 1, 1),
+                                     (13, 29, 3), (300, 270, 1)])
+def test_f32_adjoint_tiles(lbm, nx, ny, B):  # noqa: F811
+    """FP32 learned step and its adjoint (tiles of 128 consecutive nodes, two groups
+    per CTA; the last shape gives every group several): one recorded step's
+    populations, dL/dtheta and dL/df0 against FP64 torch autograd through a
+    restatement of the step, 1e-4 relative as in the adjoint's parity tests."""
+    from perf import cases as C
+    case = dict(path="train", kind="mlp_f32", tau=0.6, force=1e-3, nx=nx, ny=ny, batch=B)
+    f0 = C._populations(C._C2, C._W2, 0.03 * torch.randn(2, B, ny, nx, generator=C._gen(nx),
+                                                         device=DEV, dtype=torch.float64),
+                        C._gen(ny), 0.05)
+    theta = torch.tensor(inputs.xavier_mlp(5, bias_scale=0.3, gain=3.0, out_scale=0.02),
+                         dtype=torch.float32, device=DEV)
+    g = torch.randn((B, 9, ny, nx), generator=C._gen(3), device=DEV, dtype=torch.float64)
+    lat = lbm.Lattice(nx, ny, B, tau=0.6, force_amp=1e-3, force_mode=C.MODE_2D, device=DEV)
+    lat.set_state(f0)
+    ws = torch.empty(lat.record_bytes(1, 1) // 4, dtype=torch.float32, device=DEV)
+    w = lbm.weights_struct(theta)
+    lat.forward_record(1, 1, w, ws, "f32")
+    dW = torch.empty(lbm.LBM_MLP_NPARAMS, dtype=torch.float32, device=DEV)
+    dF = torch.empty((B, 9, ny, nx), dtype=torch.float32, device=DEV)
+    lat.backward(g.float(), w, ws, dW, dF, "f32")
+    f, th = f0.double().requires_grad_(True), theta.double().requires_grad_(True)
+    out = C._stream(C._C2, C._collide(case, C._C2, C._W2, f, "bgk", th))
+    (out * g.float().double()).sum().backward()
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())
+    assert rel(lat.get_state(), out.detach()) <= 1e-6
+    assert rel(dW, th.grad) <= 1e-4 and rel(dF, f.grad) <= 1e-4
+    assert lat.status() == lbm.LBM_OK
