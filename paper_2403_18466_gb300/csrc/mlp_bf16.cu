@@ -285,24 +285,27 @@ __device__ __forceinline__ void pull_node(const float *__restrict__ in, size_t p
 // layer reproduces BGK bit for bit; fx = 0 on a lattice without forcing, so
 // there is no branch) and rho/tau.  Returns true for an unstable node.
 struct NodePrep {
-  float base[Q];
+  Opposites base;
   float rw;
 };
-__device__ __forceinline__ bool prep_node(const float d[Q], float omega, float fx,
+__device__ __forceinline__ bool prep_node(const float f[Q], float omega, float fx,
                                           unsigned char *a1, int r, NodePrep &P) {
-  const Moments m = node_moments(d);
-  float deq[Q];
-  shifted_feq(m, deq);
-  float xin[Q];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) xin[i] = (d[i] - deq[i]) * m.inv_rho;
+  const Moments m = node_moments(f);
+  const Opposites d = pair_opposites(f), e = shifted_feq_pairs(m);
+  // n = f - feq: x = n / rho and the relaxation f - omega n
+  const float n0 = v_sub(d.r, e.r);
+  const float2 nx = v_sub(d.x, e.x), ny = v_sub(d.y, e.y), nd = v_sub(d.d, e.d),
+               na = v_sub(d.a, e.a);
+  const float2 inv = both(m.inv_rho), mo = both(-omega);
+  const float x0 = v_mul(n0, m.inv_rho);
+  const float2 xx = v_mul(nx, inv), xy = v_mul(ny, inv), xd = v_mul(nd, inv), xa = v_mul(na, inv);
   *reinterpret_cast<uint4 *>(a1 + canon_offset(r, 0, K1)) =
-      make_uint4(pack_bf16x2_alu(xin[0], xin[1]), pack_bf16x2_alu(xin[2], xin[3]),
-                 pack_bf16x2_alu(xin[4], xin[5]), pack_bf16x2_alu(xin[6], xin[7]));
+      make_uint4(pack_bf16x2_alu(x0, xx.x), pack_bf16x2_alu(xy.x, xx.y),
+                 pack_bf16x2_alu(xy.y, xd.x), pack_bf16x2_alu(xa.x, xd.y));
   *reinterpret_cast<uint4 *>(a1 + canon_offset(r, 8, K1)) =
-      make_uint4(pack_bf16x2_alu(xin[8], 1.0f), 0u, 0u, 0u);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) P.base[i] = bgk_relax(d[i], deq[i], omega);
+      make_uint4(pack_bf16x2_alu(xa.y, 1.0f), 0u, 0u, 0u);
+  P.base = {v_fma(-omega, n0, d.r), v_fma(mo, nx, d.x), v_fma(mo, ny, d.y), v_fma(mo, nd, d.d),
+            v_fma(mo, na, d.a)};
   add_edm_force_x(m, fx, P.base);
   P.rw = m.rho * omega;
   return is_unstable(m);
@@ -319,10 +322,12 @@ __device__ __forceinline__ void finish_node(const uint32_t ov[16], const NodePre
   const float sx = (o[1] - o[3]) + (o[5] - o[6]) + (o[8] - o[7]);
   const float sy = (o[2] - o[4]) + (o[5] + o[6]) - (o[7] + o[8]);
   const float k1 = -s * (1.0f / 9.0f), k2 = -sx * (1.0f / 6.0f), k3 = -sy * (1.0f / 6.0f);
+  const Opposites &b = P.base;
+  const float base[Q] = {b.r, b.x.x, b.y.x, b.x.y, b.y.y, b.d.x, b.a.x, b.d.y, b.a.y};
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const float oi = o[i] + (k1 + ((float)cx(i) * k2 + (float)cy(i) * k3));
-    out[i] = fmaf(P.rw, oi, P.base[i]);
+    out[i] = fmaf(P.rw, oi, base[i]);
   }
 }
 
