@@ -8,8 +8,6 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include "approx.cuh"
-
 namespace lbm {
 namespace d3 {
 
@@ -100,25 +98,6 @@ __device__ __forceinline__ void add_edm_force(const Moments &m, float Fx, float 
     const float cF = cdot(i, Fx, Fy, Fz), cs = cdot(i, sx, sy, sz);
     out[i] += wf(i) * (cF * (3.0f + 4.5f * cs) - Fs15);
   }
-}
-
-// Smagorinsky tau_eff = (tau0 + sqrt(tau0^2 + 18 (C_s Delta)^2 Q / rho)) / 2 with
-// Q = sqrt(2 Pi:Pi), Pi_ab = sum c_ia c_ib (f_i - feq_i) (SI section 1).
-__device__ __forceinline__ float smag_omega(const float d[Q], const float deq[Q], float inv_rho,
-                                            float tau0_sq, float tau0, float c18) {
-  float pxx = 0.f, pyy = 0.f, pzz = 0.f, pxy = 0.f, pxz = 0.f, pyz = 0.f;
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const float n = d[i] - deq[i];
-    if (cx(i)) pxx += n;
-    if (cy(i)) pyy += n;
-    if (cz(i)) pzz += n;
-    if (cx(i) && cy(i)) pxy += cx(i) * cy(i) > 0 ? n : -n;
-    if (cx(i) && cz(i)) pxz += cx(i) * cz(i) > 0 ? n : -n;
-    if (cy(i) && cz(i)) pyz += cy(i) * cz(i) > 0 ? n : -n;
-  }
-  const float pp = pxx * pxx + pyy * pyy + pzz * pzz + 2.0f * (pxy * pxy + pxz * pxz + pyz * pyz);
-  return smagorinsky_omega(pp, inv_rho, tau0, tau0_sq, c18);
 }
 
 __device__ __forceinline__ bool is_unstable(const Moments &m) {

@@ -207,3 +207,20 @@ def test_f32_adjoint_tiles(lbm, nx, ny, B):  # noqa: F811
     assert rel(lat.get_state(), out.detach()) <= 1e-6
     assert rel(dW, th.grad) <= 1e-4 and rel(dF, f.grad) <= 1e-4
     assert lat.status() == lbm.LBM_OK
+
+
+@pytest.mark.parametrize("kind", ["bgk", "smag"])
+@pytest.mark.parametrize("nx,ny,nz,B", [(1, 1, 1, 2), (2, 2, 2, 1), (129, 2, 3, 1), (5, 7, 9, 2)])
+def test_d3q19_step_strong_flow(lbm, kind, nx, ny, nz, B):  # noqa: F811
+    """D3Q19 steps on even and odd parts of opposite pairs, with every velocity
+    and force component large: 1e-5 of each weight against the oracle, as in
+    the one-step parity test."""
+    lat = lbm.Lattice3D(nx, ny, nz, B, tau=0.52, smag_cs=0.3, force_amp=3e-3, force_mode=1,
+                        device=DEV)
+    lat.set_state(_dev(field3d(B, nz, ny, nx, seed=61, neq=0.05, mean_u=(0.12, -0.15, 0.09))))
+    g = o3.stream_push(_np(lat.get_state()))
+    lat.step(1, kind)
+    prm = o3.params(0.52, smag_cs=0.3, force_amp=3e-3, force_mode=1)
+    ref = o3.stream_pull(o3.step(o3.BGK if kind == "bgk" else o3.SMAG, g, prm))
+    assert wpe(_np(lat.get_state()), ref) <= 1e-5
+    assert lat.status() == lbm.LBM_OK
