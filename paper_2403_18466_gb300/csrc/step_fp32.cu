@@ -31,14 +31,6 @@ constexpr int SCALAR_THREADS = 128;
 
 enum { KIND_BGK = 0, KIND_SMAG = 1 };
 
-// Pi^neq : Pi^neq with Pi^neq_ab = sum_i c_ia c_ib n_i, n = f - feq (SI sec. 1).
-template <class T>
-__device__ __forceinline__ T stress_norm(const T n[Q]) {
-  const T dg = v_add(v_add(n[5], n[6]), v_add(n[7], n[8]));
-  const T pxx = v_add(v_add(n[1], n[3]), dg), pyy = v_add(v_add(n[2], n[4]), dg);
-  const T pxy = v_add(v_sub(n[5], n[6]), v_sub(n[7], n[8]));
-  return v_fma(pyy, pyy, v_fma(v_mul(v_c<T>(2.0f), pxy), pxy, v_mul(pxx, pxx)));
-}
 __device__ __forceinline__ float smag_omega(float pp, float inv_rho, const CollideParams &p) {
   return smagorinsky_omega(pp, inv_rho, p.tau, p.tau0_sq, p.smag_c18);
 }
@@ -46,47 +38,89 @@ __device__ __forceinline__ float2 smag_omega(float2 pp, float2 inv_rho, const Co
   return make_float2(smag_omega(pp.x, inv_rho.x, p), smag_omega(pp.y, inv_rho.y, p));
 }
 
+__device__ __forceinline__ bool unstable(const MomentsT<float> &m, bool, bool) {
+  return is_unstable(m);
+}
+__device__ __forceinline__ bool unstable(const MomentsT<float2> &m, bool x, bool y) {
+  return is_unstable(m, x, y);
+}
+
 // Collide one node (float) or two (float2: packed f32x2, half the issue slots)
 // in place (shifted representation), add the force.  Every operation is
 // rounded explicitly, so both forms, and every kernel that uses them, give the
-// same bits.  Returns true if a node is unstable (|u| >= 0.4 or not finite).
-template <int KIND>
-__device__ __forceinline__ bool collide_node(float d[Q], const CollideParams &p, float fx) {
-  const Moments m = node_moments(d);
-  const bool bad = is_unstable(m);
-  float deq[Q];
+// same bits.  Returns true if a node is unstable (|u| >= 0.4 or not finite;
+// act_x, act_y: which of two nodes count).
+//
+// BGK: the operations of the learned kernels, which reduce to it bit for bit.
+template <class T>
+__device__ __forceinline__ bool collide_bgk(T d[Q], const CollideParams &p, T fx, bool act_x,
+                                            bool act_y) {
+  const MomentsT<T> m = node_moments(d);
+  const bool bad = unstable(m, act_x, act_y);
+  T deq[Q];
   shifted_feq(m, deq);
-  float omega = p.omega;
-  if (KIND == KIND_SMAG) {
-    float n[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) n[i] = v_sub(d[i], deq[i]);
-    omega = smag_omega(stress_norm(n), m.inv_rho, p);
-  }
-#pragma unroll
-  for (int i = 0; i < Q; ++i) d[i] = bgk_relax(d[i], deq[i], omega);
+  for (int i = 0; i < Q; ++i) d[i] = bgk_relax(d[i], deq[i], v_c<T>(p.omega));
   add_edm_force_x(m, fx, d);  // fx = 0 without forcing
   return bad;
 }
-template <int KIND>
-__device__ __forceinline__ bool collide_node(float2 d[Q], const CollideParams &p, float2 fx,
-                                             bool act_x, bool act_y) {
-  const MomentsT<float2> m = node_moments(d);
-  const bool bad = is_unstable(m, act_x, act_y);
-  float2 deq[Q];
-  shifted_feq(m, deq);
-  float2 omega = make_float2(p.omega, p.omega);
-  if (KIND == KIND_SMAG) {
-    float2 n[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) n[i] = v_sub(d[i], deq[i]);
-    omega = smag_omega(stress_norm(n), m.inv_rho, p);
-  }
-#pragma unroll
-  for (int i = 0; i < Q; ++i) d[i] = bgk_relax(d[i], deq[i], omega);
-  add_edm_force_x(m, fx, d);
+
+// Smagorinsky, on the even and odd parts s = f_i + f_opp, t = f_i - f_opp of the
+// opposite pairs (1, 3), (2, 4), (5, 7), (6, 8): feq's even part is w E with
+// E = drho - 1.5 j.u + 4.5 (c.j)(c.u) and its odd part 3 w c.j, so a pair shares E,
+// and Pi^neq_ab = sum c_a c_b (f - feq) needs the even parts alone: about two thirds
+// of the FP32 operations of the sums direction by direction.
+template <class T>
+__device__ __forceinline__ bool collide_smag(T d[Q], const CollideParams &p, T fx, bool act_x,
+                                             bool act_y) {
+  const T sx = v_add(d[1], d[3]), sy = v_add(d[2], d[4]), sd = v_add(d[5], d[7]),
+          sa = v_add(d[6], d[8]);
+  const T td = v_sub(d[5], d[7]), ta = v_sub(d[6], d[8]);
+  MomentsT<T> m;
+  m.drho = v_add(d[0], v_add(v_add(sx, sy), v_add(sd, sa)));
+  const T jx = v_add(v_sub(d[1], d[3]), v_sub(td, ta));
+  const T jy = v_add(v_sub(d[2], d[4]), v_add(td, ta));
+  m.rho = v_add(v_c<T>(1.0f), m.drho);
+  m.inv_rho = v_rcp(m.rho);
+  m.ux = v_mul(jx, m.inv_rho);
+  m.uy = v_mul(jy, m.inv_rho);
+  const bool bad = unstable(m, act_x, act_y);
+  const T xx = v_mul(jx, m.ux), yy = v_mul(jy, m.uy), c45 = v_c<T>(4.5f);
+  const T B = v_fma(v_c<T>(-1.5f), v_add(xx, yy), m.drho);
+  const T jd = v_add(jx, jy), ja = v_sub(jy, jx);
+  const T Ex = v_fma(c45, xx, B), Ey = v_fma(c45, yy, B);
+  const T Ed = v_fma(c45, v_mul(jd, v_add(m.ux, m.uy)), B);
+  const T Ea = v_fma(c45, v_mul(ja, v_sub(m.uy, m.ux)), B);
+  // tau_eff in closed form (SI sec. 1)
+  const T w1 = v_c<T>(wf(1)), w5 = v_c<T>(wf(5));
+  const T m1 = v_c<T>(-2.0f * wf(1)), m5 = v_c<T>(-2.0f * wf(5));
+  const T nd = v_fma(m5, Ed, sd), na = v_fma(m5, Ea, sa), diag = v_add(nd, na);
+  const T pxx = v_add(v_fma(m1, Ex, sx), diag), pyy = v_add(v_fma(m1, Ey, sy), diag);
+  const T pxy = v_sub(nd, na);
+  const T pp = v_fma(pyy, pyy, v_fma(v_mul(v_c<T>(2.0f), pxy), pxy, v_mul(pxx, pxx)));
+  const T omega = smag_omega(pp, m.inv_rho, p);
+  // f + omega (feq - f), feq = w (E +- 3 c.j)
+  const T three = v_c<T>(3.0f);
+  auto relax = [&](T &a, T &b, T w, T E, T cj) {
+    a = v_fma(omega, v_sub(v_mul(w, v_fma(three, cj, E)), a), a);
+    b = v_fma(omega, v_sub(v_mul(w, v_fma(v_c<T>(-3.0f), cj, E)), b), b);
+  };
+  d[0] = v_fma(omega, v_sub(v_mul(v_c<T>(wf(0)), B), d[0]), d[0]);
+  relax(d[1], d[3], w1, Ex, jx);
+  relax(d[2], d[4], w1, Ey, jy);
+  relax(d[5], d[7], w5, Ed, jd);
+  relax(d[6], d[8], w5, Ea, ja);
+  add_edm_force_x(m, fx, d);  // fx = 0 without forcing
   return bad;
 }
+
+template <int KIND, class T>
+__device__ __forceinline__ bool collide_node(T d[Q], const CollideParams &p, T fx,
+                                             bool act_x = true, bool act_y = true) {
+  return KIND == KIND_SMAG ? collide_smag(d, p, fx, act_x, act_y)
+                           : collide_bgk(d, p, fx, act_x, act_y);
+}
+
 __device__ __forceinline__ float4 ldg4(const float *p) {
   return __ldg(reinterpret_cast<const float4 *>(p));
 }
