@@ -22,7 +22,8 @@ struct lbm3d_ctx {
   cudaStream_t stream;
   Collide3 cp;
   int *d_flag;     // [0] unstable, [1] device wait timeout
-  float *d_wf32;   // transposed weights of the FP32 collision, in the allocation of d_flag
+  // in the allocation of d_flag:
+  float *d_wf32;   // transposed weights of the FP32 collision
   float *d_force;  // ny + nz + nx floats (F_x(y), F_y(z), F_z(x)), or nullptr
   void *d_wtc;     // BF16 operand tiles of the tensor-core collision (first use)
   int sms;
@@ -106,10 +107,10 @@ int lbm3d_init(lbm3d_ctx **out, const lbm3d_params *p, float *b0, float *b1, voi
     delete c;
     return LBM_ERR_CUDA;
   }
-  // flags and the FP32 collision's weight scratch (574 KB) in one allocation,
-  // made here so that a first lbm3d_step may run under stream capture
-  const size_t scratch = 256 + sizeof(float) * lbm::d3::mlp_f32_weight_floats();
-  if (cudaMalloc(&c->d_flag, scratch) != cudaSuccess ||
+  // flags, the FP32 collision's weight scratch (574 KB, here so that a first
+  // lbm3d_step may run under stream capture) and the force tables in one allocation
+  const size_t axes = (size_t)p->ny + p->nz + p->nx, wf = lbm::d3::mlp_f32_weight_floats();
+  if (cudaMalloc(&c->d_flag, 256 + sizeof(float) * (wf + axes)) != cudaSuccess ||
       cudaMemset(c->d_flag, 0, 2 * sizeof(int)) != cudaSuccess) {
     cudaFree(c->d_flag);
     delete c;
@@ -118,17 +119,16 @@ int lbm3d_init(lbm3d_ctx **out, const lbm3d_params *p, float *b0, float *b1, voi
   c->d_wf32 = reinterpret_cast<float *>(c->d_flag) + 256 / sizeof(float);
   if (p->force_amp != 0.0) {
     // sine tables in FP64 on the host, one per axis
-    std::vector<float> h((size_t)p->ny + p->nz + p->nx);
+    std::vector<float> h(axes);
     const double k = 2.0 * M_PI * (double)p->force_mode;
     for (int y = 0; y < p->ny; ++y) h[y] = (float)(p->force_amp * std::sin(k * y / p->ny));
     for (int z = 0; z < p->nz; ++z)
       h[(size_t)p->ny + z] = (float)(p->force_amp * std::sin(k * z / p->nz));
     for (int x = 0; x < p->nx; ++x)
       h[(size_t)p->ny + p->nz + x] = (float)(p->force_amp * std::sin(k * x / p->nx));
-    if (cudaMalloc(&c->d_force, sizeof(float) * h.size()) != cudaSuccess ||
-        cudaMemcpy(c->d_force, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice) !=
-            cudaSuccess) {
-      cudaFree(c->d_force);
+    c->d_force = c->d_wf32 + wf;
+    if (cudaMemcpy(c->d_force, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice) !=
+        cudaSuccess) {
       cudaFree(c->d_flag);
       delete c;
       return LBM_ERR_CUDA;
@@ -144,8 +144,7 @@ int lbm3d_init(lbm3d_ctx **out, const lbm3d_params *p, float *b0, float *b1, voi
 void lbm3d_destroy(lbm3d_ctx *c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  cudaFree(c->d_flag);
-  cudaFree(c->d_force);
+  cudaFree(c->d_flag);  // and the scratch behind it
   cudaFree(c->d_wtc);
   delete c;
 }

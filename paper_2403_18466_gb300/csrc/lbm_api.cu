@@ -24,9 +24,9 @@ struct lbm_ctx {
   int device;
   int sms;
   CollideParams cp;
-  // scratch (library-owned, device)
+  // scratch (library-owned, device); the first four in one allocation
   int *d_flag;          // [0] unstable, [1] device wait timeout, [2] bad node index
-  void *d_tiles;        // operand tiles of the tensor-core step, in the allocation of d_flag
+  void *d_tiles;        // operand tiles of the tensor-core step
   bool tiles_ready;     // they hold the weights of the call in progress
   float *d_force;       // ny floats, or nullptr
   float *d_loss_part;   // lbm::loss_partials(g) doubles (float or double partials)
@@ -203,26 +203,34 @@ int lbm_init(lbm_ctx **out, const lbm_params *p, float *f_buf0, float *f_buf1,
   c->cp.smag_c18 = (float)(18.0 * (p->smag_cs * p->smag_delta) * (p->smag_cs * p->smag_delta));
   c->cp.force = nullptr;
   int rc = LBM_OK;
-  if (cudaMalloc(&c->d_flag, 256 + lbm::mlp_bf16_tile_bytes()) != cudaSuccess ||
-      cudaMemset(c->d_flag, 0, 3 * sizeof(int)) != cudaSuccess)
+  // all scratch in one allocation: flags, the loss's partial sums, the tensor-
+  // core step's operand tiles (here, so that a first step may run under stream
+  // capture), the force table
+  auto rounded = [](size_t n) { return (n + 255) / 256 * 256; };
+  const size_t at_loss = 256;
+  const size_t at_tiles = at_loss + rounded(sizeof(double) * lbm::loss_partials(c->g));
+  const size_t at_force = at_tiles + rounded(lbm::mlp_bf16_tile_bytes());
+  const size_t bytes = at_force + (p->force_amp != 0.0 ? sizeof(float) * p->ny : 0);
+  char *scratch = nullptr;
+  if (cudaMalloc(&scratch, bytes) != cudaSuccess ||
+      cudaMemset(scratch, 0, 3 * sizeof(int)) != cudaSuccess)
     rc = LBM_ERR_CUDA;
-  c->d_tiles = reinterpret_cast<char *>(c->d_flag) + 256;
+  c->d_flag = reinterpret_cast<int *>(scratch);
+  c->d_loss_part = reinterpret_cast<float *>(scratch + at_loss);
+  c->d_tiles = scratch + at_tiles;
   if (rc == LBM_OK && p->force_amp != 0.0) {
     // F_x(y) = F0 sin(2 pi m y / ny), evaluated in double on the host
     float *h = static_cast<float *>(std::malloc(sizeof(float) * p->ny));
     if (!h) rc = LBM_ERR_ARG;
     for (int y = 0; rc == LBM_OK && y < p->ny; ++y)
       h[y] = (float)(p->force_amp * std::sin(2.0 * M_PI * (double)p->force_mode * y / p->ny));
-    if (rc == LBM_OK && (cudaMalloc(&c->d_force, sizeof(float) * p->ny) != cudaSuccess ||
-                         cudaMemcpy(c->d_force, h, sizeof(float) * p->ny,
-                                    cudaMemcpyHostToDevice) != cudaSuccess))
+    c->d_force = reinterpret_cast<float *>(scratch + at_force);
+    if (rc == LBM_OK && cudaMemcpy(c->d_force, h, sizeof(float) * p->ny, cudaMemcpyHostToDevice) !=
+                            cudaSuccess)
       rc = LBM_ERR_CUDA;
     std::free(h);
     c->cp.force = c->d_force;
   }
-  if (rc == LBM_OK &&
-      cudaMalloc(&c->d_loss_part, sizeof(double) * lbm::loss_partials(c->g)) != cudaSuccess)
-    rc = LBM_ERR_CUDA;
   if (rc != LBM_OK) {
     lbm_destroy(c);
     return rc;
@@ -235,9 +243,7 @@ void lbm_destroy(lbm_ctx *c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
   else cudaDeviceSynchronize();
-  cudaFree(c->d_flag);
-  cudaFree(c->d_force);
-  cudaFree(c->d_loss_part);
+  cudaFree(c->d_flag);  // and the scratch behind it
   cudaFree(c->d_dw_part);
   cudaFree(c->d_diag_u);
   cudaFree(c->d_diag_uh);
