@@ -92,8 +92,8 @@ typedef struct {
  * (the pull scheme stores f_post at time t; the pre-collision populations
  * at t+1 are the streamed values).  Use lbm_set_state / lbm_get_state to
  * move populations in and out.  Allocates the context and a small device
- * scratch area (status flag, force table, reduction partials), freed by
- * lbm_destroy.  Synchronous. */
+ * scratch area (status flag, force table, reduction partials, 15 KB of operand
+ * tiles for the tensor-core step), freed by lbm_destroy.  Synchronous. */
 int lbm_init(lbm_ctx **out, const lbm_params *p, float *f_buf0, float *f_buf1,
              void *cuda_stream);
 

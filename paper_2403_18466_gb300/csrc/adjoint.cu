@@ -397,8 +397,6 @@ int adjoint_blocks(const Grid &g, int sms) {
   return (int)(blocks < sms ? blocks : sms);
 }
 
-size_t adjoint_smem_bytes() { return sizeof(AdjSmem); }
-
 cudaError_t launch_adjoint_step(const Grid &g, const float *state_n, const float *lam_next,
                                 float *lam_out, const CollideParams &p, const MlpF32 &w,
                                 float *dw_partials, int rows, int accumulate, cudaStream_t s) {

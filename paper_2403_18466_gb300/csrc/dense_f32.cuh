@@ -3,9 +3,10 @@
 // f32x2 arithmetic with operands in shared memory, and an accurate tanh.
 //
 // Operands are row-major [row][k] with a row stride that is 4 or 12 modulo 32
-// floats, so that loads of consecutive rows are free of bank conflicts.  A thread sums R x C outputs, each with the sums over the even and
-// the odd inputs in one packed accumulator (adjacent inputs pair up without any
-// move), and per two inputs reads R + C 8-byte words for R C packed FMAs.
+// floats, so that loads of consecutive rows are free of bank conflicts.  A
+// thread sums R x C outputs, each with the sums over the even and the odd inputs
+// in one packed accumulator (adjacent inputs pair up without any move), and per
+// two inputs reads R + C 8-byte words for R C packed FMAs.
 #pragma once
 #include <cuda_runtime.h>
 

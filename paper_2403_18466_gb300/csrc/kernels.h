@@ -106,7 +106,6 @@ cudaError_t launch_activation(const float *a, int n, int path, float *out, cudaS
 // adjoint.cu -------------------------------------------------------------------
 // Number of CTAs (= rows of per-CTA dW partials) of the adjoint step.
 int adjoint_blocks(const Grid &g, int sms);
-size_t adjoint_smem_bytes();
 cudaError_t launch_adjoint_step(const Grid &g, const float *state_n, const float *lam_next,
                                 float *lam_out, const CollideParams &p, const MlpF32 &w,
                                 float *dw_partials, int rows, int accumulate, cudaStream_t s);

@@ -238,13 +238,14 @@ __global__ void __launch_bounds__(SCALAR_THREADS)
 // 32-bit loads (a warp reads 32 adjacent columns of a row), with no shuffles
 // and no moves to form the pairs.  Between steps the post-collision
 // populations are in shared memory, replaced in place.
-// What bounds it: the FP32 pipe and instruction issue (64 % of the slots at
-// 1024^2 Smagorinsky, ~190 instructions per computed node), no longer HBM; t = 3
-// on a 64 x 16 region recomputes 21 % of the nodes.  Measured (GB300, us per
+// What bounds it: the FP32 pipe and instruction issue, no longer HBM (55 % and
+// 64 % busy at 1024^2 Smagorinsky before its collision took the form of even and
+// odd parts); t = 3 on a 64 x 16 region recomputes 21 % of the nodes.  Measured (GB300, us per
 // step, BGK / Smagorinsky, one step per launch before):
-//   256^2   3.2 / 3.6 -> 1.6 / 1.9       512^2   4.6 / 5.0 -> 2.9 / 3.5
-//   1024^2 10.0 / 10.6 -> 8.4 / 10.4    2048^2  49.5 / 51.8 -> 30.2 / 36.6
-//   4096^2  185 / 189 -> 116 / 140      1001^2  11.0 / 12.0 -> 8.1 / 9.6
+//   256^2   3.2 / 3.6 -> 1.6 / 1.7       512^2   4.6 / 5.0 -> 2.8 / 3.2
+//   1024^2 10.0 / 10.6 -> 8.4 / 9.2     2048^2  49.5 / 51.8 -> 30.3 / 33.1
+//   4096^2  185 / 189 -> 115 / 126      1001^2  11.0 / 12.0 -> 7.9 / 8.6
+// (Smagorinsky direction by direction: 1.9, 3.5, 10.4, 36.6, 140, 9.6.)
 // t = 2 or 4, 32- or 24-row regions and other block sizes were within 15 % or
 // slower; four nodes per thread with 128-bit loads and shuffles (t = 2) reached
 // 41 us at 2048^2, the same with the next tile's cp.async copies in flight 44.
@@ -342,10 +343,11 @@ __global__ void __launch_bounds__(MT_THREADS, 3)
   }
 }
 
-// Several steps in one launch for small lattices, where the launches
-// are the cost (64^2: 2.9 us per step with one step per launch, 0.66 with 8): a block advances a tile of ts x ts nodes by t steps, the first
-// on the tile and the t - 1 nodes around it (one node per thread), each later
-// one on a ring less, between two shared-memory buffers.
+// Several steps in one launch for small lattices, where the launches are the
+// cost (64^2 BGK: 2.9 us per step with one step per launch, 0.66 with 8): a
+// block advances a tile of ts x ts nodes by t steps, the first on the tile and
+// the t - 1 nodes around it (one node per thread), each later one on a ring
+// less, between two shared-memory buffers.
 constexpr int MS_SIDE = 22;               // ts + 2 (t - 1) at most
 constexpr int MS_NODES = MS_SIDE * MS_SIDE;
 constexpr int MS_THREADS = 512;
