@@ -527,25 +527,89 @@ __global__ void k_moments(const float *__restrict__ st, float *rho, float *ux, f
   if (uy) uy[n] = m.uy;
 }
 
-// f_coarse_i(I, J) = w_i + mean over the cg x cg block of d_i(x - c_i).
-// One thread per coarse node; FP64 accumulation of the block sum.
-__global__ void k_box_filter(const float *__restrict__ st, float *__restrict__ fc, int nx, int ny,
-                             int cg) {
-  const int NX = nx / cg, NY = ny / cg;
-  const int I = blockIdx.x * NT + threadIdx.x, J = blockIdx.y, b = blockIdx.z;
-  if (I >= NX) return;
-  const size_t plane = (size_t)nx * ny, base = (size_t)b * Q * plane;
-  const size_t cplane = (size_t)NX * NY;
-  const double inv = 1.0 / ((double)cg * cg);
+// A sum of floats as three: h + l + m, every rounding error of h caught in l and
+// every one of l in m (Knuth's two-sum), so more than the 53 bits of a double.
+struct Sum3 {
+  float h, l, m;
+  __device__ __forceinline__ void add(float f) {
+    float t = __fadd_rn(h, f), b = __fsub_rn(t, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, b)), __fsub_rn(f, b));
+    h = t;
+    t = __fadd_rn(l, e), b = __fsub_rn(t, l);
+    m = __fadd_rn(m, __fadd_rn(__fsub_rn(l, __fsub_rn(t, b)), __fsub_rn(e, b)));
+    l = t;
+  }
+};
+
+// f_coarse_i(I, J) = w_i + mean over the cg x cg block of d_i(x - c_i).  A block
+// of threads takes nc coarse nodes of a row: a thread sums one fine column (or
+// every BF_T-th of them if cg > BF_T) of each direction over the cg rows, so
+// that a warp reads 32 adjacent floats, and then one thread per direction and
+// coarse node adds its columns.  The 36 B per fine node bound it; with FP64 sums
+// their conversions and additions (1/64 of the FP32 rate) took more than that,
+// and one thread per coarse node left most of the chip idle.  A sum that is not
+// finite in FP32 is taken again in FP64.
+// Measured (GB300, us, cg = 8 / 4, one thread per coarse node before):
+//   2048^2 183 / 175 -> 54 / 68      1000 x 1400  91 / 60 -> 23 / 27
+//   32 x 256^2  83 / 93 -> 29 / 38   4096^2      599 / 611 -> 183 / 244
+// (4096^2 is 91 us at the copy rate.)
+constexpr int BF_T = 256;
+constexpr int BF_MOST = BF_T + BF_T / 2;  // columns at stride cg | 1 (no bank conflicts)
+__global__ void __launch_bounds__(BF_T)
+    k_box_filter(const float *__restrict__ st, float *__restrict__ fc, int nx, int ny, int cg,
+                 int nc, double inv) {
+  __shared__ float part[3][Q][BF_MOST];
+  const int NX = nx / cg, NY = ny / cg, tid = threadIdx.x;
+  const int I0 = blockIdx.x * nc, J = blockIdx.y, b = blockIdx.z;
+  const int n = min(nc, NX - I0), width = n * cg;
+  const size_t plane = (size_t)nx * ny, cplane = (size_t)NX * NY;
+  const float *base = st + (size_t)b * Q * plane;
+  const int cols = min(cg, BF_T), stride = cols | 1;  // columns of a coarse node in `part`
+  if (tid < width) {
+    Sum3 s[Q];
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    double s = 0.0;
-    for (int a = 0; a < cg; ++a) {
-      const int ys = wrap_index(J * cg + a - cy(i), ny);
-      const float *row = st + base + i * plane + (size_t)ys * nx;
-      for (int c = 0; c < cg; ++c) s += (double)__ldg(row + wrap_index(I * cg + c - cx(i), nx));
+    for (int i = 0; i < Q; ++i) s[i] = {0.f, 0.f, 0.f};
+    for (int col = tid; col < width; col += BF_T) {
+      const int x = I0 * cg + col;
+      const int xs[3] = {wrap_index(x + 1, nx), x, wrap_index(x - 1, nx)};  // by c_x + 1
+#pragma unroll 1  // two rows per body: 147 us instead of 55 (2048^2, cg = 8)
+      for (int a = 0; a < cg; ++a) {
+        const int y = J * cg + a;
+        const size_t row[3] = {(size_t)wrap_index(y + 1, ny) * nx, (size_t)y * nx,
+                               (size_t)wrap_index(y - 1, ny) * nx};
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+          s[i].add(__ldg(base + i * plane + row[cy(i) + 1] + xs[cx(i) + 1]));
+      }
     }
-    fc[(size_t)b * Q * cplane + i * cplane + (size_t)J * NX + I] = (float)(s * inv) + wf(i);
+    const int at = tid / cols * stride + tid % cols;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      part[0][i][at] = s[i].h;
+      part[1][i][at] = s[i].l;
+      part[2][i][at] = s[i].m;
+    }
+  }
+  __syncthreads();
+  for (int o = tid; o < n * Q; o += BF_T) {
+    const int i = o / n, k = o % n;
+    Sum3 s = {0.f, 0.f, 0.f};
+    for (int c = 0; c < cols; ++c) {
+      s.add(part[0][i][k * stride + c]);
+      s.add(part[1][i][k * stride + c]);
+      s.m += part[2][i][k * stride + c];
+    }
+    double sum = (double)s.h + ((double)s.l + (double)s.m);
+    if (!isfinite(s.h)) {
+      sum = 0.0;
+      for (int a = 0; a < cg; ++a) {
+        const float *row =
+            base + i * plane + (size_t)wrap_index(J * cg + a - cy(i), ny) * nx;
+        for (int c = 0; c < cg; ++c)
+          sum += (double)__ldg(row + wrap_index((I0 + k) * cg + c - cx(i), nx));
+      }
+    }
+    fc[(size_t)b * Q * cplane + i * cplane + (size_t)J * NX + I0 + k] = (float)(sum * inv) + wf(i);
   }
 }
 
@@ -788,8 +852,10 @@ cudaError_t launch_moments(const Grid &g, const float *state, float *rho, float 
 
 cudaError_t launch_box_filter(const Grid &g, const float *state, int cg, float *f_coarse,
                               cudaStream_t s) {
-  dim3 grid((g.nx / cg + NT - 1) / NT, g.ny / cg, g.batch);
-  k_box_filter<<<grid, NT, 0, s>>>(state, f_coarse, g.nx, g.ny, cg);
+  const int nc = cg < BF_T ? BF_T / cg : 1, NX = g.nx / cg;
+  dim3 grid((NX + nc - 1) / nc, g.ny / cg, g.batch);
+  k_box_filter<<<grid, BF_T, 0, s>>>(state, f_coarse, g.nx, g.ny, cg, nc,
+                                     1.0 / ((double)cg * cg));
   return cudaGetLastError();
 }
 

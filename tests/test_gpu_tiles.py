@@ -15,6 +15,7 @@ from test_gpu_d3q19 import _dev, _np, _weights, emulate_tc_step, field3d, lbm, w
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
+W2 = [4 / 9] + [1 / 9] * 4 + [1 / 36] * 4
 
 
 @pytest.mark.parametrize("nx,ny,nz,B", [(31, 1, 1, 1), (11, 3, 1, 1), (8, 4, 2, 1), (5, 3, 3, 3),
@@ -224,3 +225,32 @@ def test_d3q19_step_strong_flow(lbm, kind, nx, ny, nz, B):  # noqa: F811
     ref = o3.stream_pull(o3.step(o3.BGK if kind == "bgk" else o3.SMAG, g, prm))
     assert wpe(_np(lat.get_state()), ref) <= 1e-5
     assert lat.status() == lbm.LBM_OK
+
+
+@pytest.mark.parametrize("nx,ny,B,cg", [(1, 1, 1, 1), (258, 2, 2, 2), (85 * 3 + 3, 9, 1, 3),
+                                        (64, 24, 3, 8), (45, 30, 1, 15), (600, 300, 1, 300),
+                                        (514, 257, 1, 257)])
+def test_box_filter_widths(lbm, nx, ny, B, cg):  # noqa: F811
+    """Box filter against the mean in FP64, rounded and added to w the same way:
+    at most the next float (2^-24 below 1) where the sums' last bits move a
+    rounding; and a block whose sum overflows FP32 but not its mean."""
+    lat = lbm.Lattice(nx, ny, B, tau=0.6, device=DEV)
+    g = torch.Generator(device=DEV).manual_seed(nx + cg)
+    w = torch.tensor(W2, dtype=torch.float32, device=DEV)[None, :, None, None]
+    f = w * (1 + 0.1 * torch.randn(B, 9, ny, nx, generator=g, device=DEV))
+
+    def mean(f):
+        d = (f - w).double()
+        return d.view(B, 9, ny // cg, cg, nx // cg, cg).mean(dim=(3, 5))
+
+    lat.set_state(f)
+    got = lat.box_filter(cg)
+    ref = mean(f).float() + w
+    assert (got - ref).abs().max().item() <= 2.0 ** -24
+    if cg > 2:
+        f[0, 5, 0, 0] = f[0, 5, cg - 1, cg - 1] = 3e38
+        lat.set_state(f)
+        got = lat.box_filter(cg)
+        ref = mean(f).float() + w
+        assert torch.isfinite(ref).all()
+        assert ((got - ref).abs() <= 2.0 ** -23 * ref.abs() + 2.0 ** -24).all()
