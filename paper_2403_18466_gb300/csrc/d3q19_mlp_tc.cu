@@ -563,8 +563,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     const uint32_t m_1lo = map_cta(smem_u32(&S.b1lo), 0), m_1hi = map_cta(smem_u32(&S.b1hi), 0),
                    m_2lo = map_cta(smem_u32(&S.b2lo), 0), m_2hi = map_cta(smem_u32(&S.b2hi), 0),
                    m_3 = map_cta(smem_u32(&S.b3), 0);
-    const uint32_t c1a = smem_u32(&S.c1a), c1b = smem_u32(&S.c1b), c2a = smem_u32(&S.c2a), c2b = smem_u32(&S.c2b),
-                   c3 = smem_u32(&S.c3), c4 = smem_u32(&S.c4);
+    const uint32_t c1a = smem_u32(&S.c1a), c1b = smem_u32(&S.c1b), c2a = smem_u32(&S.c2a),
+                   c2b = smem_u32(&S.c2b), c3 = smem_u32(&S.c3), c4 = smem_u32(&S.c4);
     uint32_t par = 0;
     bool ok = true;
     for (int t = 0; t < count && ok; ++t, par ^= 1) {

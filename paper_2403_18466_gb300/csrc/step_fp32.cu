@@ -545,10 +545,11 @@ struct Sum3 {
 // of threads takes nc coarse nodes of a row: a thread sums one fine column (or
 // every BF_T-th of them if cg > BF_T) of each direction over the cg rows, so
 // that a warp reads 32 adjacent floats, and then one thread per direction and
-// coarse node adds its columns.  The 36 B per fine node bound it; with FP64 sums
-// their conversions and additions (1/64 of the FP32 rate) took more than that,
-// and one thread per coarse node left most of the chip idle.  A sum that is not
-// finite in FP32 is taken again in FP64.
+// coarse node adds its columns.  Latency and issue of the sums bound it, next to
+// the 36 B per fine node.  FP64 sums would need two operations per value at 1/64
+// of the FP32 rate (by count about 60 us each at 2048^2), and one thread per
+// coarse node left most of the chip idle.  A sum that is not finite in FP32 is
+// taken again in FP64.
 // Measured (GB300, us, cg = 8 / 4, one thread per coarse node before):
 //   2048^2 183 / 175 -> 54 / 68      1000 x 1400  91 / 60 -> 23 / 27
 //   32 x 256^2  83 / 93 -> 29 / 38   4096^2      599 / 611 -> 183 / 244
