@@ -400,7 +400,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       constexpr uint32_t ID_LO = idesc_bf16_f32(256, NLO), ID_HI = idesc_bf16_f32(256, NHI),
                          ID_3 = idesc_bf16_f32(256, N3), ID_4 = idesc_bf16_f32(256, N4);
       const uint32_t P = tmem + TM_P;
-      bool issued = false;
       uint32_t par = 0;  // parity of tile t's events
       if (warp == MMA_WARP) {
         const uint32_t w1lo = sw + G_W1, w1hi = w1lo + R_LO * KX * 2;
@@ -421,7 +420,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
             mma_pair(P + NLO, tmem + TM_X + 8 * s, smem_desc(w1hi + 256 * s, 128, 16 * KX), ID_HI,
                      s > 0);
           commit_pair(smem_u32(&S.c1b));
-          issued = true;
           // L2, first pass: the lower half of h1 is ready before the upper one
           if (!wait_phase(smem_u32(&S.b1lo), par, err)) break;
           fence_after_sync();
@@ -451,7 +449,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 #pragma unroll
           for (int s = 0; s < NLO / 16; ++s)
             mma_pair(D3, tmem + col_h2()(s), smem_desc(w3 + 256 * s, 128, 16 * KH), ID_3, s > 0);
-          issued = true;
           if (!wait_phase(smem_u32(&S.b2hi), par, err)) break;
           fence_after_sync();
 #pragma unroll
@@ -472,15 +469,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
             mma_pair(tmem + TM_OUT, tmem + col_h3()(s), smem_desc(w4 + 256 * s, 128, 16 * K4), ID_4,
                      s > 0);
           commit_pair(smem_u32(&S.c4));
-          issued = true;
         }
       }
-      // this thread's outstanding MMAs are done before the tensor memory is freed
-      if (issued) {
-        const uint32_t bar = smem_u32(&S.drain[warp - MMA_WARP]);
-        commit_pair(bar);
-        if (!wait_done(bar)) record_error(err);
-      }
+      // both CTAs wait for this at their end
+      commit_pair(smem_u32(&S.drain[warp - MMA_WARP]));
     }
     __syncwarp();
   } else if (warp >= NODE_WARP) {
@@ -587,7 +579,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     }
   }
 
-  // ---- teardown: every role of both CTAs has left its loop (normally or on an error)
+  // ---- teardown: every role of both CTAs has left its loop (normally or on an error).
+  // The issuers' last commits arrive in both CTAs, and each CTA waits for its own
+  // copies of them: no MMA is outstanding when the tensor memory is freed, and no
+  // arrival is on its way to a CTA that has left.  (A cluster barrier orders what
+  // threads did, not the arrivals of a commit.)
+  if (tid < 3 && ok0 && !wait_done(smem_u32(&S.drain[tid]))) record_error(err);
   __syncwarp();
   fence_before_sync();
   cluster_sync();

@@ -1,0 +1,72 @@
+"""The D3Q19 tensor-core step runs on pairs of CTAs whose MMA commits arrive in
+both: a CTA must not leave while an arrival is on its way to it.  That is an
+order of asynchronous events, so the CPU test follows the kernel's source."""
+import os
+import re
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = os.path.join(ROOT, "paper_2403_18466_gb300", "csrc", "d3q19_mlp_tc.cu")
+
+
+def _block(src, start):
+    """Text of the braces that open at or after `start`, and its end."""
+    i = src.index("{", start)
+    depth = 0
+    for j in range(i, len(src)):
+        depth += {"{": 1, "}": -1}.get(src[j], 0)
+        if depth == 0:
+            return src[i:j + 1], j + 1
+    raise ValueError("unbalanced braces")
+
+
+def kernel_parts():
+    """The step kernel's body without comments, as (before the roles, code that
+    only CTA 0 runs, the rest)."""
+    src = re.sub(r"//[^\n]*", "", open(SRC).read())
+    body, _ = _block(src, src.index("k3_step_mlp_tc(const float"))
+    roles = body.index("if (warp >= MMA_WARP)")
+    issue, end = _block(body, body.index("rank == 0", roles))
+    return body[:roles], issue, body[roles:body.index(issue)] + body[end:]
+
+
+def test_both_ctas_wait_for_every_commit():
+    """Every barrier that a commit arrives at in both CTAs is waited for in code
+    that both run (CTA 1 issues no MMA, so a wait in the issuers' block is
+    CTA 0's alone)."""
+    _, issue, both = kernel_parts()
+    names = set(re.findall(r"commit_pair\(smem_u32\(&S\.(\w+)", issue))
+    assert {"c1a", "c4", "drain"} <= names
+    assert "commit_pair" not in both
+    for n in sorted(names):
+        assert re.search(rf"smem_u32\(&S\.{n}\b", both), n
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny,nz", [(5, 3, 2), (16, 8, 2), (64, 32, 20)])
+def test_back_to_back_steps_of_a_pair(nx, ny, nz):
+    """Steps that follow one another at once, from one pair of CTAs whose second
+    tile is empty to pairs on every SM, with a kernel in between that takes over
+    the shared memory: the same bits every time, no time-out."""
+    import torch
+
+    from paper_2403_18466_gb300 import inputs, lbm
+    dev = "cuda:0"
+    th = torch.tensor(inputs.xavier_mlp_widths(7, lbm.LBM3D_WIDTHS, bias_scale=0.1,
+                                               out_scale=0.001), dtype=torch.float32, device=dev)
+    w = lbm.weights3d_struct(th)
+    lat = lbm.Lattice3D(nx, ny, nz, 1, tau=0.7, device=dev)
+    g = torch.Generator(device=dev).manual_seed(nx)
+    rest = torch.tensor([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12, device=dev) \
+        .view(1, 19, 1, 1, 1) * (1 + 0.01 * torch.rand((1, 19, nz, ny, nx), generator=g, device=dev))
+    first = None
+    for _ in range(4):
+        lat.set_state(rest)
+        for _ in range(20):
+            lat.step(3, "mlp_bf16", w)
+            lat.step(1, "mlp_f32", w)
+        got = lat.get_state()
+        assert lat.status() == lbm.LBM_OK
+        first = got if first is None else first
+        assert torch.equal(got, first) and torch.isfinite(got).all()
