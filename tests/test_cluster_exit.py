@@ -1,6 +1,7 @@
 """The D3Q19 tensor-core step runs on pairs of CTAs whose MMA commits arrive in
-both: a CTA must not leave while an arrival is on its way to it.  That is an
-order of asynchronous events, so the CPU test follows the kernel's source."""
+both: a CTA must not leave while an arrival, or its own copy, is on its way to
+it.  That is an order of asynchronous events, so the CPU tests follow the
+kernel's source."""
 import os
 import re
 
@@ -41,6 +42,18 @@ def test_both_ctas_wait_for_every_commit():
     assert "commit_pair" not in both
     for n in sorted(names):
         assert re.search(rf"smem_u32\(&S\.{n}\b", both), n
+
+
+def test_weight_copy_verdict_is_common_to_the_pair():
+    """A CTA whose weights have not landed tells the other one between two
+    cluster barriers (the first: the other's error word exists; the second: the
+    verdict is read after it), and waits for its copy again before it leaves."""
+    before, _, both = kernel_parts()
+    order = r"cluster_sync\(\).*wait_done\(smem_u32\(&S\.wload\)\).*record_error\(err\).*" \
+            r"cluster_sync\(\).*ok0 = .*err"
+    assert re.search(order, before, re.S)
+    assert "S.err = 1" not in before
+    assert re.search(r"wait_done\(smem_u32\(&S\.wload\)\).*cluster_sync\(\)", both, re.S)
 
 
 @pytest.mark.gpu
