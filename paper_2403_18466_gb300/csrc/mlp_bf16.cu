@@ -558,11 +558,12 @@ __global__ void __launch_bounds__(NWG *WG_THREADS, WGS / NWG)
   }
 
   // the leader's wait gave up (the whole warpgroup left the loop together):
-  // flag it and drain the outstanding commit (full limit) before tensor
-  // memory is released
+  // flag it and wait (full limit) for what is in flight, the weights' copy or
+  // the GEMM, before shared and tensor memory are released
   if (leader && fail) {
     atomicOr(timeout_flag, 1);
-    if (count > 0) mbar_wait_bounded(bar, phase, DEFAULT_WAIT_LIMIT);
+    const bool gemm = count > 0;
+    mbar_wait_bounded(gemm ? bar : smem_u32(&S.wbar), gemm ? phase : 0, DEFAULT_WAIT_LIMIT);
   }
   flag_unstable(bad, flag);
   fence_before_sync();

@@ -1,14 +1,14 @@
-"""The D3Q19 tensor-core step runs on pairs of CTAs whose MMA commits arrive in
-both: a CTA must not leave while an arrival, or its own copy, is on its way to
-it.  That is an order of asynchronous events, so the CPU tests follow the
-kernel's source."""
+"""A CTA of a tensor-core kernel must not leave while something is on its way to
+its shared memory: its own bulk copy, or, on the CTA pairs of the D3Q19 step,
+an MMA commit of the other CTA.  That is an order of asynchronous events, so the
+CPU tests follow the kernels' source."""
 import os
 import re
 
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-SRC = os.path.join(ROOT, "paper_2403_18466_gb300", "csrc", "d3q19_mlp_tc.cu")
+CSRC = os.path.join(ROOT, "paper_2403_18466_gb300", "csrc")
 
 
 def _block(src, start):
@@ -22,11 +22,16 @@ def _block(src, start):
     raise ValueError("unbalanced braces")
 
 
+def kernel_body(name, kernel):
+    """A kernel's body without comments."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    return _block(src, src.index(kernel + "(const float"))[0]
+
+
 def kernel_parts():
-    """The step kernel's body without comments, as (before the roles, code that
-    only CTA 0 runs, the rest)."""
-    src = re.sub(r"//[^\n]*", "", open(SRC).read())
-    body, _ = _block(src, src.index("k3_step_mlp_tc(const float"))
+    """The D3Q19 step kernel's body as (before the roles, code that only CTA 0
+    runs, the rest)."""
+    body = kernel_body("d3q19_mlp_tc.cu", "k3_step_mlp_tc")
     roles = body.index("if (warp >= MMA_WARP)")
     issue, end = _block(body, body.index("rank == 0", roles))
     return body[:roles], issue, body[roles:body.index(issue)] + body[end:]
@@ -54,6 +59,42 @@ def test_weight_copy_verdict_is_common_to_the_pair():
     assert re.search(order, before, re.S)
     assert "S.err = 1" not in before
     assert re.search(r"wait_done\(smem_u32\(&S\.wload\)\).*cluster_sync\(\)", both, re.S)
+
+
+def test_late_weight_copy_of_the_2d_step_is_waited_for_at_the_exit():
+    body = kernel_body("mlp_bf16.cu", "k_step_mlp_bf16")
+    at = body.index("if (leader && fail)")
+    assert "mbar_wait_bounded" in _block(body, at)[0] and "S.wbar" in _block(body, at)[0]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(1024, 64), (1024, 704)])
+def test_time_out_in_a_call_of_several_steps(nx, ny):
+    """Steps that take their weights with a bulk copy (half-size and full CTAs):
+    a wait that runs out gives the status, and the next call is sound again.  (With
+    a tile alone on its SM one poll suffices: the thread that committed a GEMM
+    stalls at its next memory access until it is done.)"""
+    import torch
+
+    from paper_2403_18466_gb300 import inputs, lbm
+    dev = "cuda:0"
+    w = lbm.weights_struct(torch.tensor(inputs.xavier_mlp(3, out_scale=0.1), dtype=torch.float32,
+                                        device=dev))
+    g = torch.Generator(device=dev).manual_seed(ny)
+    f = torch.tensor([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4, device=dev).view(1, 9, 1, 1) * \
+        (1 + 0.01 * torch.rand((1, 9, ny, nx), generator=g, device=dev))
+    a, b = (lbm.Lattice(nx, ny, 1, tau=0.6, device=dev) for _ in range(2))
+    a.set_state(f)
+    a.set_wait_limit(1)
+    a.step(3, "mlp_bf16", w)
+    assert a.status() == lbm.LBM_ERR_TIMEOUT
+    a.set_wait_limit(0)
+    a.clear_status()
+    for lat in (a, b):
+        lat.set_state(f)
+        lat.step(3, "mlp_bf16", w)
+        assert lat.status() == lbm.LBM_OK
+    assert torch.equal(a.get_state(), b.get_state())
 
 
 @pytest.mark.gpu
