@@ -7,7 +7,7 @@
 // e = x^, y^ (periodic).  For rmax <= 256: strips of 32 lines staged in shared
 // memory with an rmax halo, one thread per separation; otherwise one block per
 // (r, chunk of rows).  Either way per-thread FP32 sums over at most 32 nodes are
-// flushed into FP64 (or FP32-pair) accumulators and per-block FP64 partials are
+// flushed into FP64 (or FP32-triple) accumulators and per-block FP64 partials are
 // added in a fixed order, so results are reproducible.
 //
 // Energy spectrum: E(k) = 1/2 sum_{round(|k'|) = k} |u_hat(k')|^2 / N^2 for the
@@ -91,24 +91,27 @@ __global__ void __launch_bounds__(SF_THREADS)
 // [column][y].  Nine FMA-pipe operations per increment for its six powers
 // bound the kernel.  Each lane sums 32 terms, adjacent in x, in FP32 (S^1 is the
 // rounding left of a sum that cancels, so the order is part of the result)
-// before they go into its running sum, a pair of FP32 numbers kept by
-// error-free additions (about 48 bits): FP64 additions, at 1/64 of the FP32
-// rate, took as long as all the rest.
-// Measured (GB300, 1024^2, r <= 256, E(k) and S^p(r) together): 0.34 ms, 1.04
-// before (this kernel 295 us with two blocks per SM, 0.37 ms in all).
+// before they go into its running sum, three FP32 numbers kept by error-free
+// additions (more than the 53 bits of a double): FP64 additions, at 1/64 of the
+// FP32 rate, took as long as all the rest.
+// Measured (GB300, 1024^2, r <= 256, E(k) and S^p(r) together): 0.36 ms, 1.04
+// before; 0.34 ms with pairs of FP32 numbers (48 bits).
 constexpr int SFT_R = 256;    // largest separation
 constexpr int SF_LINES = 32;
 constexpr int SF_STRIDE = SF_LINES + 4;  // of a position of the x increments
 constexpr int SF_MOST_BLOCKS = 4096;
 
-// (hi, lo) += f without rounding error but in lo (Knuth's two-sum)
-__device__ __forceinline__ void pair_add(float2 &hi, float2 &lo, float2 f) {
+// (h, l, m) += f: every rounding error of h caught in l and every one of l in m
+// (Knuth's two-sum), per lane.
+__device__ __forceinline__ float2 two_sum(float2 &a, float2 f) {
   const float2 m1 = make_float2(-1.f, -1.f);
-  const float2 s = __fadd2_rn(hi, f);
-  const float2 b = __ffma2_rn(hi, m1, s);
-  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(b, m1, s), m1, hi), __ffma2_rn(b, m1, f));
-  lo = __fadd2_rn(lo, e);
-  hi = s;
+  const float2 s = __fadd2_rn(a, f), b = __ffma2_rn(a, m1, s);
+  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(b, m1, s), m1, a), __ffma2_rn(b, m1, f));
+  a = s;
+  return e;
+}
+__device__ __forceinline__ void sum3_add(float2 &h, float2 &l, float2 &m, float2 f) {
+  m = __fadd2_rn(m, two_sum(l, two_sum(h, f)));
 }
 
 // a modulo n, n <= a < 2 n in the usual case
@@ -152,9 +155,9 @@ __global__ void __launch_bounds__(SFT_R, 3)
       strip[l * ystride + j] = l < lw ? u[(size_t)periodic(p0 + j, ny) * nx] : 0.f;
   }
   __syncthreads();
-  float2 hi[6], lo[6];
+  float2 hi[6], lo[6], lo2[6];
 #pragma unroll
-  for (int p = 0; p < 6; ++p) hi[p] = lo[p] = make_float2(0.f, 0.f);
+  for (int p = 0; p < 6; ++p) hi[p] = lo[p] = lo2[p] = make_float2(0.f, 0.f);
   const float2 m1 = make_float2(-1.f, -1.f);
   auto add = [](float2 (&f)[6], float2 d) {
     const float2 d2 = __fmul2_rn(d, d), d3 = __fmul2_rn(d2, d);
@@ -184,8 +187,8 @@ __global__ void __launch_bounds__(SFT_R, 3)
         }
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
-          pair_add(hi[p], lo[p], f[0][p]);
-          pair_add(hi[p], lo[p], f[1][p]);
+          sum3_add(hi[p], lo[p], lo2[p], f[0][p]);
+          sum3_add(hi[p], lo[p], lo2[p], f[1][p]);
         }
       }
     } else {
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(SFT_R, 3)
           add(f, d);
         }
 #pragma unroll
-        for (int p = 0; p < 6; ++p) pair_add(hi[p], lo[p], f[p]);
+        for (int p = 0; p < 6; ++p) sum3_add(hi[p], lo[p], lo2[p], f[p]);
       }
     }
   }
@@ -212,7 +215,8 @@ __global__ void __launch_bounds__(SFT_R, 3)
   bool finite = true;
 #pragma unroll
   for (int p = 0; p < 6; ++p) {
-    acc[p] = ((double)hi[p].x + (double)hi[p].y) + ((double)lo[p].x + (double)lo[p].y);
+    acc[p] = ((double)hi[p].x + (double)hi[p].y) +
+             (((double)lo[p].x + (double)lo[p].y) + ((double)lo2[p].x + (double)lo2[p].y));
     finite &= isfinite(acc[p]);
   }
   if (!finite && slice < slices && r <= rmax) {
