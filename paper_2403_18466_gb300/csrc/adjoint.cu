@@ -30,7 +30,7 @@
 // writes its own row of partial sums, and a second kernel adds the rows in a
 // fixed order, so dtheta is bitwise reproducible.
 // Measured (GB300): a training step of 8 x 256^2 trajectories, 16 steps, from
-// 17.3 to 11.7 ms with the forward of mlp_f32.cu (one node per thread, 128
+// 17.3 to 11.9 ms with the forward of mlp_f32.cu (one node per thread, 128
 // threads per SM, before).
 #include "adjoint_node.cuh"
 #include "dense_f32.cuh"
@@ -173,11 +173,12 @@ __global__ void __launch_bounds__(THREADS, 1)
       float *dst = (layer == 1 ? &G.h1[ng][0] : &G.h2[ng][0]) + ug;
 #pragma unroll
       for (int c = 0; c < 8; c += 2) {
-        const float b0 = layer == 1 ? 0.f : S.b2[c * 8 + ug];
-        const float b1 = layer == 1 ? 0.f : S.b2[c * 8 + 8 + ug];
+        const float2 bias = layer == 1 ? make_float2(0.f, 0.f)
+                                       : make_float2(S.b2[c * 8 + ug], S.b2[c * 8 + 8 + ug]);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-          const float2 h = tanh2(make_float2(total(acc[r][c]) + b0, total(acc[r][c + 1]) + b1));
+          const float2 h =
+              tanh2(__fadd2_rn(make_float2(total(acc[r][c]), total(acc[r][c + 1])), bias));
           dst[r * 16 * HS + c * 8] = h.x;
           dst[r * 16 * HS + c * 8 + 8] = h.y;
         }

@@ -12,12 +12,11 @@
 // force update, the layers are matrix products over the tile (8 nodes x 8 units
 // per thread, dense_f32.cuh), and the activations stay in shared memory, each
 // layer's in place of its input's.
-// Measured (GB300): 3.08 G nodes/s at 2048^2, 2.85 at 4 x 333 x 250, 31 us per
-// step at 256^2 and 15 at 64^2, against 3.01, 2.03, 96 and 90 with one node per
+// Measured (GB300): 3.00 G nodes/s at 2048^2, 2.73 at 4 x 333 x 250, 33 us per
+// step at 256^2 and 16 at 64^2, against 3.01, 2.03, 96 and 90 with one node per
 // thread and tanhf; FMA pipe ~60 % busy.  The error of the learned correction
-// against 64 bits fell from 1.9e-7 to 1.2 - 1.5e-7.  tanh2 against tanhf, errors
-// in units of 2^-24 relative: [-9, 9] rms 0.33 and 0.43, maximum 2.5 and 3.2;
-// |x| < 0.8 rms 0.45 and 1.01; 0.8 .. 3.8 rms 0.37 and 0.35, maximum 2.6 and 2.2.
+// against 64 bits fell from 1.9e-7 to 1.2 - 1.5e-7.  (tanh2's accuracy and what
+// it costs stand beside it.)
 #include "dense_f32.cuh"
 #include "kernels.h"
 
@@ -125,11 +124,12 @@ __global__ void __launch_bounds__(TILE, BLOCKS_PER_SM)
       if (layer == 2) __syncthreads();  // h1 is read
 #pragma unroll
       for (int c = 0; c < 8; c += 2) {
-        const float b0 = layer == 1 ? 0.f : S.b2[c * 8 + ug];
-        const float b1 = layer == 1 ? 0.f : S.b2[c * 8 + 8 + ug];
+        const float2 bias = layer == 1 ? make_float2(0.f, 0.f)
+                                       : make_float2(S.b2[c * 8 + ug], S.b2[c * 8 + 8 + ug]);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-          const float2 h = tanh2(make_float2(total(acc[r][c]) + b0, total(acc[r][c + 1]) + b1));
+          const float2 h =
+              tanh2(__fadd2_rn(make_float2(total(acc[r][c]), total(acc[r][c + 1])), bias));
           S.h[r * 16 + ng][c * 8 + ug] = h.x;
           S.h[r * 16 + ng][c * 8 + 8 + ug] = h.y;
         }
