@@ -17,6 +17,9 @@
 // from the adjacent lane by a warp shuffle, and only the warp's edge lanes
 // (and the periodic wrap) issue an extra scalar load.  Stores are aligned
 // 128-bit.  Other widths take a one-node-per-thread kernel.
+#include <algorithm>
+#include <cmath>
+
 #include "approx.cuh"
 #include "kernels.h"
 #include "lattice.cuh"
@@ -808,14 +811,37 @@ __global__ void k_shift(const float *__restrict__ in, float *__restrict__ out, i
 
 }  // namespace
 
-// Up to 128^2 nodes a step is shorter than its launch: 8 steps per launch on
-// 8 x 8 tiles, mostly recomputed rings, take 0.7 us per step at 64^2 and 1.2 at
-// 128^2 (the tile kernel 1.4 and 1.4, one step per launch 3.0 and 2.7); at 256^2
-// they take 2.6 us against 1.6.  Planes of 2^31 nodes or more (beyond the tile
-// kernel's 32-bit offsets) go step by step.
+// Steps per launch: whichever of the three forms has the least estimated time per
+// step, from the sizes alone.  The estimates are fits to measurements (GB300, us
+// per step; 60 shapes of 4 k to 4 M nodes, within about 25 % of them):
+//   single steps  2.4 (4-node threads; 1.5 one-node) plus 8 ps per node in L2, 10
+//                 one-node, 11.6 from HBM, and at least 2.4 (1.1) ns per block, of 512
+//                 (128) nodes of one row: narrow lattices have many blocks;
+//   k_steps_tile  t = 3: 1.0 + 0.54 per wave of one region per SM, 5.2 ns per region
+//                 beyond three; a region stores 60 x 12 nodes, and computes 64 x 16
+//                 however few of them the lattice has;
+//   k_steps_small t = 8: 0.6 + 1.9 ns per 8 x 8 tile, up to 128^2 nodes.
+// So squares and batches of small lattices take several steps per launch (64^2: 2.9
+// -> 0.7 us per step, 256 lattices of 64^2: 40 -> 15, 64 x 16384: 40 -> 13), and
+// lattices a row or two high do not: 65536 x 2 takes 3.5 us by single steps and 6.1 by
+// the tile kernel, 16384 x 1 takes 3.0, 2.6 and (small kernel) 4.2.  The tile kernel has
+// to be 5 % better: with equal estimates (61 x 1000) its Smagorinsky form is slower.
+// Plane offsets of all forms are 32-bit (lbm_init refuses planes of 2^31 nodes).
 StepPlan step_plan(const Grid &g) {
-  if (g.nodes() <= 128 * 128) return {8, 8};
-  if (g.plane() < 1u << 31) return {MT_MOST, 0};
+  const double nodes = (double)g.nodes(), rows = (double)g.ny * g.batch;
+  auto over = [](int n, int d) { return (double)((n + d - 1) / d); };
+  const bool vec = g.nx % 4 == 0;
+  const double per_node = nodes > 1.5e6 ? 11.6e-6 : (vec ? 8e-6 : 10e-6);
+  const double single = std::max((vec ? 2.4 : 1.5) + per_node * nodes,
+                                 vec ? 2.4e-3 * over(g.nx, 4 * VEC_THREADS) * rows
+                                     : 1.1e-3 * over(g.nx, SCALAR_THREADS) * rows);
+  constexpr int RING = 2 * (MT_MOST - 1), TS = 8;
+  const double regions = over(g.nx, MT_X - RING) * over(g.ny, MT_Y - RING) * g.batch;
+  const double waves = std::ceil(regions / 152);
+  const double tile = std::max(1.0 + 0.54 * std::min(waves, 3.0), 5.2e-3 * regions);
+  const double small = 0.6 + 1.9e-3 * over(g.nx, TS) * over(g.ny, TS) * g.batch;
+  if (nodes <= 128 * 128 && small <= single && small <= tile) return {8, TS};
+  if (1.05 * tile <= single) return {MT_MOST, 0};
   return {1, 0};
 }
 
