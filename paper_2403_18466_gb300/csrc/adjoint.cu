@@ -401,16 +401,11 @@ int adjoint_blocks(const Grid &g, int sms) {
 cudaError_t launch_adjoint_step(const Grid &g, const float *state_n, const float *lam_next,
                                 float *lam_out, const CollideParams &p, const MlpF32 &w,
                                 float *dw_partials, int rows, int accumulate, cudaStream_t s) {
-  static bool attr_set = false;  // per-process; the attribute is per function
-  const size_t smem = sizeof(AdjSmem);
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_adjoint_step,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  k_adjoint_step<<<rows, THREADS, smem, s>>>(state_n, lam_next, lam_out, g.nx, g.ny,
-                                             (long long)g.nodes(), p, w, dw_partials, accumulate);
+  const cudaError_t e = allow_smem(k_adjoint_step, sizeof(AdjSmem));
+  if (e != cudaSuccess) return e;
+  k_adjoint_step<<<rows, THREADS, sizeof(AdjSmem), s>>>(state_n, lam_next, lam_out, g.nx, g.ny,
+                                                        (long long)g.nodes(), p, w, dw_partials,
+                                                        accumulate);
   return cudaGetLastError();
 }
 

@@ -803,13 +803,8 @@ cudaError_t launch_adjoint_tc(const Grid &g, const float *state_n, const float *
                               float *lam_out, const CollideParams &p, const MlpF32 &w,
                               float *dw_partials, int rows, int accumulate, int *timeout_flag,
                               cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_adjoint_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  const cudaError_t e = allow_smem(k_adjoint_tc, SMEM_BYTES);
+  if (e != cudaSuccess) return e;
   if ((long long)g.nx * g.ny * g.batch * Q >= (1LL << 31)) return cudaErrorInvalidValue;
   // a programmatic dependent of the previous kernel on the stream: in the
   // backward pass that is always one of this library's (the push, a recompute

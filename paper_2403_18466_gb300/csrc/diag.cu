@@ -372,16 +372,11 @@ cudaError_t launch_structure_functions(const Grid &g, const float *ux, const flo
                                        double *part, double *S, cudaStream_t s) {
   if (sf_tiled(g, rmax)) {
     const SfShape sh = sf_shape(g);
-    static bool attr_set = false;
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(k_sf_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sf_smem(256, SFT_R));
-      if (e != cudaSuccess) return e;
-      attr_set = true;
-    }
+    cudaError_t e = allow_smem(k_sf_strips, sf_smem(256, SFT_R));  // the largest
+    if (e != cudaSuccess) return e;
     k_sf_strips<<<sh.bx + sh.by, SFT_R, sf_smem(sh.h, rmax), s>>>(ux, uy, g.nx, g.ny, g.batch,
                                                                      rmax, sh, part);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_sum_rows<<<(6 * rmax + 31) / 32, 32 * SUM_SLICES, 0, s>>>(
         part, sh.bx + sh.by, 6 * rmax, 1.0 / (2.0 * (double)g.nodes()), S);

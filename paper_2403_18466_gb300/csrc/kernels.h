@@ -27,6 +27,16 @@ struct MlpF32 {
   const float *w1, *b1, *w2, *b2, *w3, *b3;
 };
 
+// Lets `kern` take `bytes` of dynamic shared memory (more than 48 KB has to be
+// asked for).  The attribute belongs to the current device's copy of the kernel,
+// so it is set at every launch (0.2 us of host time beside the launch's 1.5)
+// instead of being remembered.  The same size every time: another thread may be
+// about to launch the same kernel.
+template <class K>
+inline cudaError_t allow_smem(K *kern, size_t bytes) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // step_fp32.cu ---------------------------------------------------------------
 // Plain collisions: a launch advances t steps, 1 <= t <= step_plan(g).steps;
 // tile: side of the small-lattice kernel's tiles, 0 for the others.
@@ -72,8 +82,9 @@ cudaError_t launch_push(const Grid &g, const float *in, float *out, cudaStream_t
 cudaError_t launch_pull(const Grid &g, const float *in, float *out, cudaStream_t s);
 
 // mlp_f32.cu -------------------------------------------------------------------
+// sms: streaming multiprocessors of the device (of both learned steps).
 cudaError_t launch_step_mlp_f32(const Grid &g, const float *in, float *out,
-                                const CollideParams &p, const MlpF32 &w, int *flag,
+                                const CollideParams &p, const MlpF32 &w, int sms, int *flag,
                                 cudaStream_t s);
 
 // mlp_bf16.cu ------------------------------------------------------------------
@@ -93,8 +104,8 @@ cudaError_t launch_prepare_weights_bf16(const MlpPtrs &w, int dtype, void *tiles
 // dependent of it (its prologue overlaps that kernel's last tiles).
 cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,
                                  const CollideParams &p, const MlpPtrs &w, int dtype,
-                                 const void *tiles, int *flag, int *timeout_flag, cudaStream_t s,
-                                 unsigned wait_limit = 0, int max_ctas = 0, bool chain = false);
+                                 const void *tiles, int sms, int *flag, int *timeout_flag,
+                                 cudaStream_t s, unsigned wait_limit = 0, int max_ctas = 0, bool chain = false);
 
 // Compiled layout of the tensor-core step: tile warpgroups per SM and, of
 // every 8 activation pairs, how many the XU evaluates.

@@ -120,12 +120,13 @@ cudaError_t one_step(lbm_ctx *c, const float *in, float *out, lbm_collision kind
     case LBM_SMAG:
       return lbm::launch_steps_smag(c->g, in, out, c->cp, steps, c->d_flag, c->stream);
     case LBM_MLP_F32:
-      return lbm::launch_step_mlp_f32(c->g, in, out, c->cp, f32_view(w), c->d_flag, c->stream);
+      return lbm::launch_step_mlp_f32(c->g, in, out, c->cp, f32_view(w), c->sms, c->d_flag,
+                                      c->stream);
     case LBM_MLP_BF16: {
       return lbm::launch_step_mlp_bf16(c->g, in, out, c->cp, ptrs(w), w->dtype,
-                                       c->tiles_ready ? c->d_tiles : nullptr, c->d_flag,
-                                       c->d_flag + 1, c->stream, c->wait_limit, c->max_ctas,
-                                       chain);
+                                       c->tiles_ready ? c->d_tiles : nullptr, c->sms,
+                                       c->d_flag, c->d_flag + 1, c->stream, c->wait_limit,
+                                       c->max_ctas, chain);
     }
   }
   return cudaErrorInvalidValue;

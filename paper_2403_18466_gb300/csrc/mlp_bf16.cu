@@ -626,16 +626,8 @@ cudaError_t launch_prepare_weights_bf16(const MlpPtrs &w, int dtype, void *tiles
 
 cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,
                                  const CollideParams &p, const MlpPtrs &w, int dtype,
-                                 const void *tiles, int *flag, int *timeout_flag, cudaStream_t s,
-                                 unsigned wait_limit, int max_ctas, bool chain) {
-  static int sms = 0;
-  static bool attr_done[4] = {false, false, false, false};
-  if (!sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+                                 const void *tiles, int sms, int *flag, int *timeout_flag,
+                                 cudaStream_t s, unsigned wait_limit, int max_ctas, bool chain) {
   const long long count = (long long)((g.nx + WG_THREADS - 1) / WG_THREADS) * g.ny * g.batch;
   // Few tiles and prepared weights: the half-size CTAs (up to four tiles per SM,
   // all in flight at once either way; 256^2: 7.8 -> 7.3 us per step).
@@ -646,12 +638,8 @@ cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,
               : src == 2 ? k_step_mlp_bf16<2, WGS>
                          : k_step_mlp_bf16<2, FEW_WGS>;
   const size_t smem = few ? smem_bytes<FEW_WGS>() : smem_bytes<WGS>();
-  if (!attr_done[src]) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_done[src] = true;
-  }
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
   // One CTA per SM while there are tiles for it: a tile alone on its SM is done
   // sooner than eight at a time (64^2: 9.3 -> 5.0 us per step).
   long long ctas = count;

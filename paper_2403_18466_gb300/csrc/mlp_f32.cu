@@ -162,19 +162,11 @@ __global__ void __launch_bounds__(TILE, BLOCKS_PER_SM)
 }  // namespace
 
 cudaError_t launch_step_mlp_f32(const Grid &g, const float *in, float *out,
-                                const CollideParams &p, const MlpF32 &w, int *flag,
+                                const CollideParams &p, const MlpF32 &w, int sms, int *flag,
                                 cudaStream_t s) {
-  static int slots = 0;
-  if (!slots) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaFuncSetAttribute(k_step_mlp_f32,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(Smem));
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    slots = BLOCKS_PER_SM * sms;
-  }
+  const cudaError_t e = allow_smem(k_step_mlp_f32, sizeof(Smem));
+  if (e != cudaSuccess) return e;
+  const long long slots = (long long)BLOCKS_PER_SM * sms;
   const long long nodes = (long long)g.nodes(), tiles = (nodes + TILE - 1) / TILE;
   k_step_mlp_f32<<<(unsigned)(tiles < slots ? tiles : slots), TILE, sizeof(Smem), s>>>(
       in, out, g.nx, g.ny, nodes, p, w, flag);

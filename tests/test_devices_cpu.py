@@ -1,0 +1,74 @@
+"""The library's host code on two devices of one process, over a runtime without
+GPUs (fake_cudart.cpp): every entry point that works on the first works on the
+second."""
+import ctypes as C
+import glob
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_2403_18466_gb300 import build, lbm
+    cxx, inc = shutil.which("g++"), "/usr/local/cuda/include"
+    if not cxx or not os.path.exists(os.path.join(inc, "cuda_runtime_api.h")):
+        pytest.skip("no C++ compiler or CUDA headers")
+    build.build()
+    out = str(tmp_path_factory.mktemp("fake") / "liblbm_fake.so")
+    subprocess.run([cxx, "-shared", "-fPIC", "-O1", "-I", inc, "-o", out,
+                    os.path.join(HERE, "fake_cudart.cpp"),
+                    *sorted(glob.glob(os.path.join(build.BUILD, "*.o")))], check=True)
+    lib = C.CDLL(out)
+    for name, (res, args) in lbm._SIGS.items():
+        getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
+    return lib
+
+
+def _calls(lib, lbm, mem):
+    """(name, status) of a pass over the entry points that launch kernels."""
+    ctx, c3 = C.c_void_p(), C.c_void_p()
+    prm = lbm.make_params(64, 48, 1, tau=0.6, smag_cs=0.1, force_amp=1e-4, force_mode=1)
+    p = [C.addressof(m) for m in mem]
+    w = lbm.lbm_weights(*[p[2]] * 6, 0)
+    yield "init", lib.lbm_init(C.byref(ctx), C.byref(prm), p[0], p[1], None)
+    yield "set_state", lib.lbm_set_state(ctx, p[2])
+    for kind in lbm.KINDS.values():
+        for n in (1, 4):
+            yield f"step {kind} {n}", lib.lbm_step(ctx, n, kind, C.byref(w))
+    size = lib.lbm_record_bytes(C.byref(prm), 3, 2)
+    for rec, back in (("lbm_forward_record", "lbm_backward"),
+                      ("lbm_forward_record_bf16", "lbm_backward_bf16")):
+        yield rec, getattr(lib, rec)(ctx, 3, 2, C.byref(w), p[3], size)
+        yield back, getattr(lib, back)(ctx, p[2], C.byref(w), p[3], size, p[4], None)
+    yield "structure", lib.lbm_structure_functions(ctx, 20, p[4])
+    yield "structure", lib.lbm_structure_functions(ctx, 300, p[4])
+    yield "spectrum", lib.lbm_energy_spectrum(ctx, 20, p[4])
+    yield "box", lib.lbm_box_filter(ctx, 4, p[4])
+    large = lbm.make_params(1024, 700, 1, tau=0.6)  # more than four tiles per SM
+    big = C.c_void_p()
+    yield "init", lib.lbm_init(C.byref(big), C.byref(large), p[0], p[1], None)
+    yield "step", lib.lbm_step(big, 4, lbm.LBM_MLP_BF16, C.byref(w))
+    prm3 = lbm.lbm3d_params(8, 8, 8, 1, 0.6, 0.1, 1.0, 0.0, 0, 0)
+    w3 = lbm.lbm3d_weights(*[p[2]] * 8, 0)
+    yield "init 3d", lib.lbm3d_init(C.byref(c3), C.byref(prm3), p[0], p[1], None)
+    for kind in lbm.KINDS.values():
+        yield f"step 3d {kind}", lib.lbm3d_step(c3, 2, kind, C.byref(w3))
+    for c in (ctx, big):
+        lib.lbm_destroy(c)
+    lib.lbm3d_destroy(c3)
+
+
+def test_second_device_of_a_process(lib):
+    from paper_2403_18466_gb300 import lbm
+    mem = [(C.c_char * n)() for n in (1 << 22, 1 << 22, 1 << 22, 1 << 24, 1 << 18)]
+    before = lib.fake_launches()
+    for device in (0, 1):
+        lib.fake_set_device(device)
+        bad = [(name, rc) for name, rc in _calls(lib, lbm, mem) if rc != lbm.LBM_OK]
+        assert not bad, f"device {device}: {bad}"
+    assert lib.fake_launches() - before > 80
