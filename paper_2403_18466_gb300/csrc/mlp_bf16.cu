@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(NWG *WG_THREADS, WGS / NWG)
   // the GEMM, before shared and tensor memory are released
   if (leader && fail) {
     atomicOr(timeout_flag, 1);
-    const bool gemm = count > 0;
+    const bool gemm = SRC < 2 || count > 0;
     mbar_wait_bounded(gemm ? bar : smem_u32(&S.wbar), gemm ? phase : 0, DEFAULT_WAIT_LIMIT);
   }
   flag_unstable(bad, flag);
