@@ -879,6 +879,9 @@ cudaError_t launch_moments(const Grid &g, const float *state, float *rho, float 
 
 cudaError_t launch_box_filter(const Grid &g, const float *state, int cg, float *f_coarse,
                               cudaStream_t s) {
+  // a block of one node is that node: the same values in half the time (1024^2: 126 us
+  // as sums; 88 with one thread per coarse node)
+  if (cg == 1) return launch_subsample(g, state, cg, f_coarse, s);
   const int nc = cg < BF_T ? BF_T / cg : 1, NX = g.nx / cg;
   dim3 grid((NX + nc - 1) / nc, g.ny / cg, g.batch);
   k_box_filter<<<grid, BF_T, 0, s>>>(state, f_coarse, g.nx, g.ny, cg, nc,
