@@ -374,8 +374,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   cluster_sync();  // both CTAs run, and their error words are set up
   // the weights have landed (bounded; every thread polls, so that all see the copy);
   // if a CTA's have not, neither CTA starts its roles
-  const bool loaded = wait_done(smem_u32(&S.wload));
-  if (!loaded) record_error(err);
+  if (!wait_done(smem_u32(&S.wload))) record_error(err);
   cluster_sync();
   fence_after_sync();
   const uint32_t tmem = S.taddr;
@@ -588,8 +587,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   // arrival is on its way to a CTA that has left.  (A cluster barrier orders what
   // threads did, not the arrivals of a commit.)
   if (tid < 3 && ok0 && !wait_done(smem_u32(&S.drain[tid]))) record_error(err);
-  // a copy that was late is waited for once more, so that none is in flight at the exit
-  if (tid == 0 && !loaded) wait_done(smem_u32(&S.wload));
+  // (a copy that was late is waited for once more, so that none is in flight at the exit)
+  if (tid == 0) wait_done(smem_u32(&S.wload));
   __syncwarp();
   fence_before_sync();
   cluster_sync();
