@@ -1,32 +1,34 @@
 """The library's host code on two devices of one process, over a runtime without
 GPUs (fake_cudart.cpp): every entry point that works on the first works on the
-second."""
+second.
+
+The pointers are the host's, so no call may reach the real runtime, which torch puts
+in the process's global symbol scope: the library binds its calls to the runtime it
+was linked with (-Bsymbolic) and leaves none open (-z defs), and it runs in a process
+of its own, without torch and without a visible device."""
 import ctypes as C
 import glob
 import os
 import shutil
 import subprocess
-
-import pytest
+import sys
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
-@pytest.fixture(scope="module")
-def lib(tmp_path_factory):
-    from paper_2403_18466_gb300 import build, lbm
+def fake_library(folder):
+    import pytest
+
+    from paper_2403_18466_gb300 import build
     cxx, inc = shutil.which("g++"), "/usr/local/cuda/include"
     if not cxx or not os.path.exists(os.path.join(inc, "cuda_runtime_api.h")):
         pytest.skip("no C++ compiler or CUDA headers")
     build.build()
-    out = str(tmp_path_factory.mktemp("fake") / "liblbm_fake.so")
-    subprocess.run([cxx, "-shared", "-fPIC", "-O1", "-I", inc, "-o", out,
-                    os.path.join(HERE, "fake_cudart.cpp"),
+    out = os.path.join(folder, "liblbm_fake.so")
+    subprocess.run([cxx, "-shared", "-fPIC", "-O1", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-I", inc,
+                    "-o", out, os.path.join(HERE, "fake_cudart.cpp"),
                     *sorted(glob.glob(os.path.join(build.BUILD, "*.o")))], check=True)
-    lib = C.CDLL(out)
-    for name, (res, args) in lbm._SIGS.items():
-        getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
-    return lib
+    return out
 
 
 def _calls(lib, lbm, mem):
@@ -63,8 +65,12 @@ def _calls(lib, lbm, mem):
     lib.lbm3d_destroy(c3)
 
 
-def test_second_device_of_a_process(lib):
+def two_devices(path):
     from paper_2403_18466_gb300 import lbm
+    assert "torch" not in sys.modules and os.environ["CUDA_VISIBLE_DEVICES"] == ""
+    lib = C.CDLL(path)
+    for name, (res, args) in lbm._SIGS.items():
+        getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
     mem = [(C.c_char * n)() for n in (1 << 22, 1 << 22, 1 << 22, 1 << 24, 1 << 18)]
     before = lib.fake_launches()
     for device in (0, 1):
@@ -72,3 +78,16 @@ def test_second_device_of_a_process(lib):
         bad = [(name, rc) for name, rc in _calls(lib, lbm, mem) if rc != lbm.LBM_OK]
         assert not bad, f"device {device}: {bad}"
     assert lib.fake_launches() - before > 80
+
+
+def test_second_device_of_a_process(tmp_path):
+    import torch  # noqa: F401  (the real runtime in this process must not matter)
+    env = {**os.environ, "CUDA_VISIBLE_DEVICES": "", "PYTHONPATH": os.path.dirname(HERE)}
+    run = subprocess.run([sys.executable, os.path.abspath(__file__), fake_library(str(tmp_path))],
+                         env=env, capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr
+
+
+
+if __name__ == "__main__":
+    two_devices(sys.argv[1])
