@@ -420,14 +420,8 @@ cudaError_t launch_steps(const Grid &g, const float *in, float *out, const Colli
   cfg.numAttrs = 1;
   const StepPlan plan = step_plan(g);
   if (t > 1 && plan.tile > 0) {
-    static bool attr_done = false;
-    const int smem = 2 * Q * MS_NODES * (int)sizeof(float);
-    if (!attr_done) {
-      const cudaError_t e = cudaFuncSetAttribute(
-          k_steps_small<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      attr_done = true;
-    }
+    constexpr size_t smem = 2 * Q * MS_NODES * sizeof(float);
+    static_assert(smem <= 48 * 1024, "what a launch may take without asking");
     cfg.gridDim = dim3((g.nx + plan.tile - 1) / plan.tile, (g.ny + plan.tile - 1) / plan.tile,
                        g.batch);
     cfg.blockDim = dim3(MS_THREADS);
@@ -435,14 +429,8 @@ cudaError_t launch_steps(const Grid &g, const float *in, float *out, const Colli
     return cudaLaunchKernelEx(&cfg, k_steps_small<KIND>, in, out, g.nx, g.ny, plan.tile, t, p, flag);
   }
   if (t > 1) {
-    static bool attr_done = false;
-    const int smem = Q * MT_Y * MT_X * (int)sizeof(float);
-    if (!attr_done) {
-      const cudaError_t e = cudaFuncSetAttribute(
-          k_steps_tile<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      attr_done = true;
-    }
+    constexpr size_t smem = Q * MT_Y * MT_X * sizeof(float);
+    static_assert(smem <= 48 * 1024, "what a launch may take without asking");
     const int tw = MT_X - 2 * (t - 1), th = MT_Y - 2 * (t - 1);
     cfg.gridDim = dim3((g.nx + tw - 1) / tw, (g.ny + th - 1) / th, g.batch);
     cfg.blockDim = dim3(MT_THREADS);

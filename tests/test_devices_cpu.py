@@ -9,6 +9,7 @@ of its own, without torch and without a visible device."""
 import ctypes as C
 import glob
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -87,6 +88,17 @@ def test_second_device_of_a_process(tmp_path):
                          env=env, capture_output=True, text=True, timeout=300)
     assert run.returncode == 0, run.stderr
 
+
+def test_launchers_hold_no_state_of_the_process():
+    """A variable that outlives a launch would be one for all devices and threads
+    (noalloc.cu keeps its buffers by device, under a lock)."""
+    from paper_2403_18466_gb300 import build
+    for src in build._sources() + build._headers():
+        if os.path.basename(src) == "noalloc.cu":
+            continue
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(src).read(), flags=re.S)
+        held = re.findall(r"\bstatic (?!constexpr\b|const\b)[^;({]*[=;]", text)
+        assert not held, f"{os.path.basename(src)}: {held}"
 
 
 if __name__ == "__main__":
