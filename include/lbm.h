@@ -149,7 +149,7 @@ int lbm_set_wait_limit(lbm_ctx *ctx, unsigned polls);
 
 /* Launch shape of the tensor-core step (no counterpart in the paper): caps
  * the persistent grid of LBM_MLP_BF16 steps at n CTAs for the later lbm_step
- * calls of this context (0, the default, restores one CTA per SM).  With
+ * calls of this context (0, the default, restores at most one per SM).  With
  * fewer CTAs each warpgroup walks more tiles, so a lattice small enough for
  * an element-by-element check against a reference still exercises the
  * kernel's tile-to-tile path (staging the next tile, crossing row and

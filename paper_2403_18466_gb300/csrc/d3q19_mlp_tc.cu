@@ -42,8 +42,8 @@
 // N = 112 and 32 below it), 68 per tile; the rest of a tile's ~9.6 k cycles is
 // the hop from L3 over L1 to L2 (a commit reaches its waiters ~700 cycles after
 // the last MMA) and the drains, which share the tensor memory with the MMAs.
-// Measured (GB300): 4.0 G nodes/s at 128^3 and 192^3 (1,020 TFLOP/s), 3.56 at
-// 64^3, where one CTA per tile of a row with W2 streamed ran at 2.68, 2.05 and
+// Measured (GB300): 4.0 G nodes/s at 256^3 (1,020 TFLOP/s), 3.9 at 128^3, 3.49 at
+// 64^3, where one CTA per tile of a row with W2 streamed ran at 2.74, 2.68 and
 // 1.29 G nodes/s.
 //
 // Roles in a CTA of 480 threads (one CTA per SM, a cluster persistent over a

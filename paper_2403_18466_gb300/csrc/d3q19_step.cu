@@ -101,8 +101,8 @@ __device__ __forceinline__ float along(float ax, float ay, float az) {  // c . a
 // and the EDM term (Eq. S5) has even part w (4.5 (c.F)(c.s_F) - 1.5 F.s_F),
 // s_F = 2 u + F/rho, and odd part 3 w c.F: little more than half the operations of
 // a sum direction by direction.  The weights multiply last: with 3 w as a rounded
-// constant the momentum drifted by its error in every step (4.7e-8 instead of
-// 3.4e-8 relative after 20 steps).  Returns true if the node is unstable.
+// constant the momentum drifted by its error in every step (error against 64 bits
+// after 20 steps at 128^3 4.7e-8 instead of 3.1e-8).  Returns true if the node is unstable.
 template <int KIND>
 __device__ __forceinline__ bool collide_pairs(float d[Q], const Collide3 &c, float Fx, float Fy,
                                               float Fz) {

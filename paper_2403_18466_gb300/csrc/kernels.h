@@ -99,7 +99,7 @@ cudaError_t launch_prepare_weights_bf16(const MlpPtrs &w, int dtype, void *tiles
 // tiles: the prepared weights, or nullptr to lay them out in every CTA.
 // wait_limit: polls of each bounded mbarrier wait before the kernel gives up
 // and sets *timeout_flag (0 = the default, 2^20); max_ctas: cap on the
-// persistent grid (0 = one CTA per SM); chain: the previous operation on `s`
+// persistent grid (0 = at most as many as SMs); chain: the previous operation on `s`
 // is this kernel with the same weights, so it is launched as a programmatic
 // dependent of it (its prologue overlaps that kernel's last tiles).
 cudaError_t launch_step_mlp_bf16(const Grid &g, const float *in, float *out,

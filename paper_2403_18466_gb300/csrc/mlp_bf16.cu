@@ -444,8 +444,9 @@ __global__ void __launch_bounds__(NWG *WG_THREADS, WGS / NWG)
   // launch this CTA may be running while the previous step (which writes `in`
   // and reads `out`) finishes on other SMs: wait for it before the first
   // access to either state buffer, and let the next step start its own
-  // prologue as SMs free up (a CTA holds all of an SM's registers, so the
-  // next step's CTA becomes resident only after this one exits).
+  // prologue as SMs free up (a CTA of WGS warpgroups holds all of an SM's
+  // registers, so the next step's becomes resident only after it exits; of
+  // FEW_WGS, two fit).
   griddep_wait();
   griddep_launch_dependents();
 
